@@ -1492,6 +1492,7 @@ wvl_status wvl_wait_timeouts(unsigned* count) {
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceSynchronize");
     e = emu_take_timeouts(count);
+    if (e == cudaSuccess) e = overlap_take_timeouts(count);
     if (e != cudaSuccess) return cuda_fail(e, "timeout counter");
     return *count ? fail(WVL_ETIMEOUT, "%u bounded device waits gave up", *count) : WVL_OK;
 }

@@ -249,6 +249,12 @@ struct PartTasks {
     }
 };
 cudaError_t launch_reduce_parts_multi(const PartTasks& t, cudaStream_t st);
+// scalar products on the tensor cores (overlap_mma.cu): workspace bytes and launch;
+// bounded waits that ran out since the last call are added to *count
+size_t overlap_mma_ws(int na, int nb, long long len, bool sym);
+cudaError_t launch_overlap_mma(int prec, int na, const void* a, int nb, const void* b, long long len,
+                               bool sym, double* S, void* ws, cudaStream_t st);
+cudaError_t overlap_take_timeouts(unsigned* count);
 // E_loc = sum_o occ (ekin + epot) into *out (one fixed-order CTA), and
 // dV = gbar rho in the potential's precision (the adjoint of E_loc in V).
 cudaError_t launch_eloc_total(const double* occ, const double* ekin, const double* epot,
