@@ -79,3 +79,19 @@ def test_rows_without_a_scale(W, dt):
     _check(S[np.ix_(keep, keep)], a[keep], a[keep])
     if dt == "float32":
         assert abs(S[12, 12] / ref[12, 12] - 1.0) < 1e-14
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-25, 1e25])
+@pytest.mark.parametrize("n,length", [(1, 3), (3, 1000), (2, 8193), (700, 40)])
+def test_dot_fp32_ranges(W, n, length, scale):
+    """FP32 products inside and outside the range of the split sums: FP64
+    rounding of a sum of at most 64 terms per thread, 256 threads and 64 blocks."""
+    import torch
+    rng = np.random.default_rng(length)
+    a = (rng.uniform(-1.0, 1.0, (n, length)) * scale).astype("float32")
+    b = (rng.uniform(-1.0, 1.0, (n, length)) * scale).astype("float32")
+    d = W.dot(torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda()).cpu().numpy()
+    a, b = a.astype(np.float64), b.astype(np.float64)
+    for o in range(0, n, max(1, n // 3)):
+        ref = O.scalar_products(a[o:o + 1], b[o:o + 1])[0, 0]
+        assert abs(d[o] - ref) <= 384 * 2.0 ** -53 * np.abs(a[o] * b[o]).sum()
