@@ -215,6 +215,15 @@ template <typename T>
 cudaError_t launch_pcg(int which, const PcgParams& q, T* a, T* b, T* c, T* d, const T* e,
                        const double* s1, const double* s2, cudaStream_t st);
 
+// The preconditioner in FP32 by the separable operator (helmholtz.cu), ncg >= 1
+// iterations: buf = five arrays of norb P floats, scal = three of norb doubles, part =
+// partials of norb x 64 and of norb x ceil(N1 N2 / 32) doubles.
+bool helmholtz_pcg_ok(const int Nf[3], int norb);
+cudaError_t launch_helmholtz_pcg(const int Nf[3], const double hg[3], const double diag[8], int norb,
+                                 const float* g, const double* eps, int ncg, float* x, double* rr,
+                                 float* const buf[5], double* const scal[3], double* const part[2],
+                                 cudaStream_t st);
+
 // Kernel-launch counter behind wvl_kernel_launches().
 void count_launches(unsigned long long k);
 // Status with a detail string for wvl_last_error() (thread-local), and its reset.
