@@ -946,6 +946,11 @@ static wvl_status run_fused(int op, std::vector<CellRun<T>>& runs, Prof* prof, c
                 // the kinetic taps are per launch: one axis spacing per launch
                 if (k > 0 && (r.hg[0] != r0.hg[0] || r.hg[1] != r0.hg[1] || r.hg[2] != r0.hg[2]))
                     break;
+                const bool plane = prog == FZ_SKM12 || prog == FZ_MFTA12;
+                // one launch shape per launch of a plane kernel
+                const FzShape shape = fz_plane_shape<T>(r.Nf[0], r.Nf[1], (long long)r.norb * r.Nf[2]);
+                if (k > 0 && plane && shape != p.shape) break;
+                p.shape = shape;
                 FzSeg<T>& s = p.seg[k];
                 s.P = r.P;
                 s.N1 = r.Nf[0];
@@ -958,7 +963,6 @@ static wvl_status run_fused(int op, std::vector<CellRun<T>>& runs, Prof* prof, c
                 s.ncb = (s.N1 + LTC - 1) / LTC;
                 const int ctiles = s.N2 * s.ncb;
                 const int ktiles = s.N3 + (s.N2 / 2) * s.ncb;   // Ekin partials per orbital
-                const bool plane = prog == FZ_SKM12 || prog == FZ_MFTA12;
                 s.RS = plane ? fz_plane_rs<T>(s.N1) : LTC;
                 long long units = r.norb;
                 T* const A = r.buf[0];

@@ -382,8 +382,8 @@ __device__ __forceinline__ void col_item(const T* __restrict__ src, const int* _
 template <int PROG>
 __host__ __device__ constexpr int fz_cthreads() { return PROG == FZ_TA3 ? 2 * FZ_CTHREADS : FZ_CTHREADS; }
 
-template <typename T, int PROG>
-__global__ void __launch_bounds__(FZ_PTHREADS)
+template <typename T, int PROG, int REGS>
+__global__ void __maxnreg__(REGS)
 fz_plane_kernel(const __grid_constant__ FzParams<T> p) {
     constexpr int VEC = 16 / (int)sizeof(T);
     constexpr int RC = FZ_RC;
@@ -405,7 +405,7 @@ fz_plane_kernel(const __grid_constant__ FzParams<T> p) {
     const int ncv = N1 / VEC;
     const int nitems = (N2 / RC) * ncv;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int NWARP = FZ_PTHREADS / 32;
+    const int NWARP = (int)(blockDim.x >> 5);
 
     // the plane, row I2 -> X + I2 RS (a warp per row, lanes over its vectors)
     {
@@ -929,7 +929,7 @@ constexpr bool fz_is_plane() { return PROG == FZ_SKM12 || PROG == FZ_MFTA12; }
 
 constexpr int FZ_SMEM_OPTIN = 224 * 1024;   // under the opt-in limit with the static reduction buffer
 
-template <typename T, int PROG>
+template <typename T, int PROG, int REGS>
 cudaError_t fz_ensure_attr() {
     static std::atomic<unsigned long long> done{0};
     int dev = 0;
@@ -938,7 +938,7 @@ cudaError_t fz_ensure_attr() {
     const unsigned long long bit = 1ull << (dev & 63);
     if (!(done.load() & bit)) {
         if constexpr (fz_is_plane<PROG>())
-            err = cudaFuncSetAttribute(fz_plane_kernel<T, PROG>,
+            err = cudaFuncSetAttribute(fz_plane_kernel<T, PROG, REGS>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, FZ_SMEM_OPTIN);
         else
             err = cudaFuncSetAttribute(fz_col_kernel<T, PROG>,
@@ -949,31 +949,46 @@ cudaError_t fz_ensure_attr() {
     return cudaSuccess;
 }
 
-template <typename T, int PROG>
-cudaError_t fz_launch(const FzParams<T>& p, size_t smem, cudaStream_t st) {
-    cudaError_t err = fz_ensure_attr<T, PROG>();
+template <typename T, int PROG, int REGS>
+cudaError_t fz_plane_launch(const FzParams<T>& p, int threads, size_t smem, cudaStream_t st) {
+    cudaError_t err = fz_ensure_attr<T, PROG, REGS>();
     if (err != cudaSuccess) return err;
-    if (p.njobs <= 0) return cudaSuccess;
-    if (p.njobs > 0x7fffffffLL || smem > (size_t)FZ_SMEM_OPTIN) return cudaErrorInvalidConfiguration;
-    if constexpr (fz_is_plane<PROG>() && sizeof(T) == 4) {
-        // the row passes' tap pairs (the slots and filters of the row passes
-        // in fz_plane_kernel)
-        FzParams<T> q = p;
-        if constexpr (PROG == FZ_SKM12) {
-            tap_pairs<K_SYN>(q.tap[0], q.tp[0]);
-            tap_pairs<K_KIN>(q.tap[1], q.tp[1]);
-            tap_pairs<K_MF>(q.tap[3], q.tp[3]);
-        } else {
-            tap_pairs<K_MFT>(q.tap[0], q.tp[0]);
-            tap_pairs<K_ANA>(q.tap[1], q.tp[1]);
-        }
-        fz_plane_kernel<T, PROG><<<dim3((unsigned)p.njobs), dim3(FZ_PTHREADS), smem, st>>>(q);
-    } else if constexpr (fz_is_plane<PROG>())
-        fz_plane_kernel<T, PROG><<<dim3((unsigned)p.njobs), dim3(FZ_PTHREADS), smem, st>>>(p);
-    else
-        fz_col_kernel<T, PROG><<<dim3((unsigned)p.njobs), dim3(fz_cthreads<PROG>()), smem, st>>>(p);
+    fz_plane_kernel<T, PROG, REGS><<<dim3((unsigned)p.njobs), dim3(threads), smem, st>>>(p);
     count_launches(1);
     return cudaGetLastError();
+}
+
+template <typename T, int PROG>
+cudaError_t fz_launch(const FzParams<T>& p, size_t smem, cudaStream_t st) {
+    if (p.njobs <= 0) return cudaSuccess;
+    if (p.njobs > 0x7fffffffLL || smem > (size_t)FZ_SMEM_OPTIN) return cudaErrorInvalidConfiguration;
+    if constexpr (fz_is_plane<PROG>()) {
+        const FzShape s = p.shape;
+        if constexpr (sizeof(T) == 4) {
+            // the row passes' tap pairs (the slots and filters of the row passes
+            // in fz_plane_kernel)
+            FzParams<T> q = p;
+            if constexpr (PROG == FZ_SKM12) {
+                tap_pairs<K_SYN>(q.tap[0], q.tp[0]);
+                tap_pairs<K_KIN>(q.tap[1], q.tp[1]);
+                tap_pairs<K_MF>(q.tap[3], q.tp[3]);
+            } else {
+                tap_pairs<K_MFT>(q.tap[0], q.tp[0]);
+                tap_pairs<K_ANA>(q.tap[1], q.tp[1]);
+            }
+            if (s.regs == 96) return fz_plane_launch<T, PROG, 96>(q, s.threads, smem, st);
+            if (s.regs == 112) return fz_plane_launch<T, PROG, 112>(q, s.threads, smem, st);
+            return fz_plane_launch<T, PROG, 128>(q, s.threads, smem, st);
+        } else {
+            return fz_plane_launch<T, PROG, 255>(p, s.threads, smem, st);
+        }
+    } else {
+        cudaError_t err = fz_ensure_attr<T, PROG, 0>();
+        if (err != cudaSuccess) return err;
+        fz_col_kernel<T, PROG><<<dim3((unsigned)p.njobs), dim3(fz_cthreads<PROG>()), smem, st>>>(p);
+        count_launches(1);
+        return cudaGetLastError();
+    }
 }
 
 }  // namespace
@@ -1007,11 +1022,20 @@ cudaError_t launch_fused(int prog, const FzParams<T>& p, size_t smem, cudaStream
 template <typename T>
 cudaError_t prepare_fused_kernels() {
     cudaError_t e;
-    if ((e = fz_ensure_attr<T, FZ_SYN3>()) != cudaSuccess) return e;
-    if ((e = fz_ensure_attr<T, FZ_SKM12>()) != cudaSuccess) return e;
-    if ((e = fz_ensure_attr<T, FZ_POT3>()) != cudaSuccess) return e;
-    if ((e = fz_ensure_attr<T, FZ_MFTA12>()) != cudaSuccess) return e;
-    return fz_ensure_attr<T, FZ_TA3>();
+    if ((e = fz_ensure_attr<T, FZ_SYN3, 0>()) != cudaSuccess) return e;
+    if ((e = fz_ensure_attr<T, FZ_POT3, 0>()) != cudaSuccess) return e;
+    if ((e = fz_ensure_attr<T, FZ_TA3, 0>()) != cudaSuccess) return e;
+    if constexpr (sizeof(T) == 8) {
+        if ((e = fz_ensure_attr<T, FZ_SKM12, 255>()) != cudaSuccess) return e;
+        return fz_ensure_attr<T, FZ_MFTA12, 255>();
+    } else {
+        if ((e = fz_ensure_attr<T, FZ_SKM12, 96>()) != cudaSuccess) return e;
+        if ((e = fz_ensure_attr<T, FZ_SKM12, 112>()) != cudaSuccess) return e;
+        if ((e = fz_ensure_attr<T, FZ_SKM12, 128>()) != cudaSuccess) return e;
+        if ((e = fz_ensure_attr<T, FZ_MFTA12, 96>()) != cudaSuccess) return e;
+        if ((e = fz_ensure_attr<T, FZ_MFTA12, 112>()) != cudaSuccess) return e;
+        return fz_ensure_attr<T, FZ_MFTA12, 128>();
+    }
 }
 
 template size_t fz_smem<float>(int, int, int, int);

@@ -121,7 +121,7 @@ enum FzProg {
     FZ_TA3 = 4,     // column, two I2 rows: H psi = A3 (w' + T3 a) (Ekin part), compressed
     FZ_NPROG = 5
 };
-constexpr int FZ_PTHREADS = 256;   // plane kernels
+constexpr int FZ_PTHREADS = 512;   // plane kernels: most threads (fz_plane_shape)
 constexpr int FZ_CTHREADS = 128;   // column kernels
 constexpr int FZ_RR = 8;           // row-pass outputs per thread (along the row)
 constexpr int FZ_RC = 8;           // column-pass outputs per thread (along the column)
@@ -153,11 +153,18 @@ struct FzSeg {
     int RS;               // shared-memory row stride in elements
 };
 
+// Threads and register cap of a plane kernel (fz_plane_shape).
+struct FzShape {
+    int threads, regs;
+    bool operator!=(const FzShape& o) const { return threads != o.threads || regs != o.regs; }
+};
+
 template <typename T>
 struct FzParams {
     T tap[4][2][32];      // the program's filters, per output parity (see fused_kernel.cu)
     float2 tp[4][32];     // FP32 row passes: tap pairs of outputs 2m, 2m + 1 (fused_kernel.cu)
     long long njobs;
+    FzShape shape;        // plane kernels: one launch shape per launch
     int nseg;
     FzSeg<T> seg[MAXSEG];
 };
@@ -170,6 +177,35 @@ inline int fz_plane_rs(int N1) {
     int w = (N1 + v - 1) / v;
     if ((w & 1) == 0) ++w;
     return w * v;
+}
+// Threads and register cap of a plane kernel, by the CTAs whose two planes fit in an
+// SM's shared memory.  FP32, microseconds of SYN3 + SKM12 / MFTA12 per call of 64 orbitals
+// (48 at 128^2, 128 at 64^2, 256 at 48^2, 512 at 32^2):
+//   one CTA       512 threads, 128 registers: 128^2 812 / 432 (256 threads 825 / 463), 120^2
+//                 770 / 413 (840 / 465)
+//   two           256; 320 at 96 registers where that saves a second round of column items
+//                 (96^2, 288 items: 456 / 219 against 460 / 236); 112^2 706 / 355, where
+//                 320 takes 720 / 345
+//   three         160: 88^2 376 / 187 (256: 391 / 202)
+//   four and more 128, at 96 registers from five on: 80^2 279 / 136 (309 / 158), 64^2
+//                 267 / 123 (310 / 163); fewer where a plane has fewer items: 48^2 315 / 146
+//                 (403 / 230), 32^2 150 / 78 (345 / 225)
+// More planes per SM overlap one's loads and barriers with another's filters.  A CTA's
+// warps are a multiple of four where CTAs share an SM's registers closely (288 threads
+// at 112 registers leave one CTA per SM: 579 / 338).  Launches of at most two CTAs per SM keep
+// 256 threads: there a plane's own time counts.  FP64 planes are bound by the FP64 pipe.
+template <typename T>
+inline FzShape fz_plane_shape(int N1, int N2, long long planes) {
+    if (sizeof(T) == 8) return {256, 255};
+    if (planes <= 2 * 152) return {256, 128};
+    const int smem = 2 * N2 * fz_plane_rs<T>(N1) * (int)sizeof(T) + 2048;
+    const int ctas = 227 * 1024 / smem;
+    const int items = (N2 / FZ_RC) * (N1 * (int)sizeof(T) / 16);
+    if (ctas <= 1) return {512, 128};
+    if (ctas == 2) return items > 256 && items <= 320 ? FzShape{320, 96} : FzShape{256, 128};
+    if (ctas == 3) return {160, 128};
+    if (ctas == 4) return {128, 128};
+    return {items <= 32 ? 32 : items <= 112 ? 64 : 128, 96};
 }
 template <typename T>
 size_t fz_smem(int prog, int N1, int N2, int N3);
