@@ -343,6 +343,14 @@ static wvl_status exec_call(PassCall<T>& c, const Tune& tn, cudaStream_t st) {
                                                       c.segs[first + q].Nf[2] / 2, s.norb, s.P, st);
                     if (e != cudaSuccess) return cuda_fail(e, "line exponent launch");
                 }
+            for (int q = 0; q < k; ++q) {
+                const Seg<T>& s = p.seg[q];
+                if (s.gin == nullptr) continue;
+                // (the exponents lie behind the scales of the two passes, build_calls)
+                const int* top = s.gmax + 3 * (s.norb * (s.P / 2));
+                cudaError_t e = launch_group_max(top, s.gmax, s.n, (long long)s.norb * (s.nsrc / s.n), st);
+                if (e != cudaSuccess) return cuda_fail(e, "line scale launch");
+            }
             cudaError_t e = launch_emu_t(c.kind, c.mode, p, blk, st);
             if (e == cudaErrorInvalidValue)
                 return fail(WVL_EUNSUPPORTED, "tensor-core pass: filter digit schedule not supported");
@@ -428,7 +436,7 @@ static size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 // tiles of LT_MIN lines, or 128-line tiles x 32-output windows when emulated
 static long long tiles_max(const int Nf[3]) {
     long long N = (long long)Nf[1] * Nf[0];
-    const long long emu_tiles = (N + emu::M - 1) / emu::M * ((Nf[2] + emu::NMIN - 1) / emu::NMIN);
+    const long long emu_tiles = (N + emu::M - 1) / emu::M * ((Nf[2] + emu::NWIN - 1) / emu::NWIN);
     return std::max((N + LT_MIN - 1) / LT_MIN, emu_tiles);
 }
 
@@ -758,6 +766,27 @@ static std::vector<PassCall<T>> build_calls(int op, std::vector<CellRun<T>>& run
             return d;
         });
         break;
+    }
+    // Tensor-core passes of one operator hand integers with a scale per line to the next
+    // pass instead of FP64 numbers (emu_kernel.cu).  Scales and exponents lie in buffer C,
+    // free outside the kinetic passes: four arrays of at most P / 2 ints per orbital
+    // (the synthesis' line exponents, then the groups' largest exponents; the scales of
+    // passes 1 and 2; the lines' exponents).
+    for (size_t i = 0; i + 1 < calls.size(); ++i) {
+        PassCall<T>&c = calls[i], &d = calls[i + 1];
+        if (!c.emu || c.kind == K_KIN || d.kind != c.kind || d.pass != c.pass + 1) continue;
+        if (!emu_hands_over(c.kind)) continue;   // (never, for the filters of the method)
+        for (size_t k = 0; k < runs.size(); ++k) {
+            int n, N;
+            pass_dims(runs[k].Nf, c.pass, n, N);
+            const long long slot = runs[k].norb * (runs[k].P / 2);
+            int* const g = reinterpret_cast<int*>(B(runs[k], C_));
+            c.segs[k].s.gout = g + c.pass * slot;
+            c.segs[k].s.gtop = g + 3 * slot;
+            d.segs[k].s.gin = g + c.pass * slot;
+            d.segs[k].s.gmax = g;
+            d.segs[k].s.nsrc = N;
+        }
     }
     return calls;
 }

@@ -38,8 +38,7 @@ namespace emu {
 constexpr int THREADS = 256;     // 8 warps: slicing 16 lines each; epilogue 32 lines x N/2 outputs
 constexpr int WARPS = THREADS / 32;
 constexpr int M = 128;           // lines per tile (MMA M, TMEM lanes)
-constexpr int NMAX = 32;         // outputs per window (MMA N), largest kind
-constexpr int NMIN = 16;
+constexpr int NWIN = 16;         // outputs per window (MMA N)
 constexpr int S = 6;             // digits per operand
 constexpr int DBITS = 10;        // bits per digit
 constexpr int DMAX = 8;          // highest diagonal kept
@@ -62,9 +61,13 @@ constexpr int TSHIFT = 20;
 // sum_t f_t x_t = T' 2^(E_x + E_f - OUT_EXP)
 constexpr int OUT_EXP = 2 * QBITS - DBITS * (2 * S - DMAX) - TSHIFT;
 
-// outputs per window, input positions read (window start o - HA, 8-aligned)
-__host__ __device__ constexpr int window_n(int kind) { return kind == K_KIN ? 16 : 32; }
-__host__ __device__ constexpr int window_k(int kind) { return 48; }
+// outputs per window, input positions read (window start o - HA, 8-aligned).  16
+// outputs read 32 positions of a 16-tap filter: 58 KB of planes, three CTAs per SM
+// (32 outputs, 98 KB and two CTAs took 31.2 instead of 29.2 ms per headline step);
+// the kinetic filter's 48 positions leave two.
+__host__ __device__ constexpr int window_n(int) { return NWIN; }
+__host__ __device__ constexpr int window_k(int kind) { return kind == K_KIN ? 48 : 32; }
+__host__ __device__ constexpr int min_ctas(int kind) { return kind == K_KIN ? 2 : 3; }
 __host__ __device__ constexpr int window_ha(int kind) { return kind == K_KIN ? 16 : 8; }
 // The filter operand holds the S digit planes side by side along N, then a
 // zero block: per 8-position chunk, rows (output j of digit fp) at fp N + j,
@@ -75,8 +78,11 @@ __host__ __device__ constexpr int lbo_b(int kind) { return (S + 1) * window_n(ki
 __host__ __device__ constexpr int tmem_cols(int kind) { return MAXACC * window_n(kind); }
 __host__ __device__ constexpr int plane_a_bytes(int kind, int mode) { return window_k(kind) / 8 * lboa(mode); }
 __host__ __device__ constexpr int b_bytes(int kind) { return window_k(kind) / 8 * lbo_b(kind); }
+// raw inputs of the next slab, 16 bytes x 4 rows per thread (not synthesis pass 1, which
+// gathers its inputs)
+__host__ __device__ constexpr int raw_bytes(int mode) { return mode == M_UNCOMP ? 0 : 4 * THREADS * 16; }
 __host__ __device__ constexpr int smem_bytes(int kind, int mode) {
-    return S * plane_a_bytes(kind, mode) + b_bytes(kind);
+    return S * plane_a_bytes(kind, mode) + b_bytes(kind) + raw_bytes(mode);
 }
 
 // Schedule of one launch: which (filter digit p, data digit q) pairs go to
@@ -92,6 +98,7 @@ struct Sched {
     unsigned char pp[MAXPAIR], pq[MAXPAIR], pacc[MAXPAIR];
     int shift[MAXACC];
     float wlow[MAXACC];
+    int tbits;               // |T'| < 2^tbits
 };
 
 struct Params {
@@ -122,14 +129,27 @@ __host__ __device__ inline long long quantize(double x, int E) {
     const int e = (int)((b >> 52) & 0x7FF);
     if (e == 0) return 0;
     // x = m 2^(e - 1075), m < 2^53 -> X = m 2^-(sh), sh = E + 1075 - QBITS - e
-    // >= -6 (e <= E + 1022).  With the mantissa shifted left by 6 first
-    // (m6 < 2^59), X is one right shift by r = sh + 6 >= 0, rounded half up
-    // on the magnitude (none of m survives once r >= 60)
-    const unsigned long long m6 = ((b & ((1ULL << 52) - 1)) | (1ULL << 52)) << 6;
+    // >= -6 (e <= E + 1022).  With the mantissa shifted left by 7 first
+    // (m7 < 2^60), 2 X is one right shift by r = sh + 6 >= 0, rounded half up
+    // on the magnitude by the last step (none of m survives once r >= 60)
+    const unsigned long long m7 = ((b & ((1ULL << 52) - 1)) | (1ULL << 52)) << 7;
     int r = E + 1081 - QBITS - e;
     r = r < 0 ? 0 : (r > 63 ? 63 : r);
-    const long long X = (long long)((m6 + ((1ULL << r) >> 1)) >> r);   // m6 + half < 2^63
+    const long long X = (long long)(((m7 >> r) + 1) >> 1);
     return (b >> 63) ? -X : X;
+}
+
+// Y = X + DBIAS >= 0 of a quantised X: its 10-bit fields, from the lowest, are the digits
+// 5 .. 1 plus 512, and what is above bit 50 is digit 0 plus 512
+constexpr long long DBIAS = 512LL * (1 + (1LL << 10) + (1LL << 20) + (1LL << 30) + (1LL << 40) + (1LL << 50));
+
+// X + DBIAS for X = round(t 2^(g + QBITS - E)), an integer t of scale 2^g (the output
+// of the pass before), |t| < 2^60, |t| 2^g <= 2^E, E - g >= HAND_MIN: one arithmetic shift
+// of 8 t, rounded half up
+constexpr int HAND_MIN = QBITS - 2;
+__host__ __device__ inline long long requantize(long long t, int g, int E) {
+    const int sh = E - HAND_MIN - g;
+    return ((t * 8 >> (sh > 63 ? 63 : sh)) + (2 * DBIAS + 1)) >> 1;
 }
 
 // signed base-1024 digits, most significant first: d[0] in [-512, 512],
@@ -196,11 +216,14 @@ inline bool build_sched(const double (&f)[2][32], int nt, Sched& s) {
             ++s.npairs;
         }
     }
+    // the kernels join the two top diagonals in 32 bits
+    if ((sabs[0] * 1024.0 + sabs[0] + sabs[1]) * 512.0 >= 2147483648.0) return false;
     // the kernels take the canonical schedule: accumulator a holds diagonal
     // a + 2, exact for a < NEXACT (shift >= 10), FP32-summed otherwise
     if (s.nacc != NACC || s.nexact != NEXACT) return false;
     for (int a = 0; a < NACC; ++a)
         if (s.shift[a] != DBITS * (DMAX - 2 - a) - TSHIFT) return false;
+    s.tbits = std::max(QBITS + 1, (int)std::ceil(std::log2(tbound)));
     return tbound < std::ldexp(1.0, 62);
 }
 
@@ -208,36 +231,33 @@ inline bool build_sched(const double (&f)[2][32], int nt, Sched& s) {
 #include <cuda_fp16.h>
 
 // The digits of two inputs, as digits() gives them, digit q of both as one
-// FP16x2 word (X0's in the low half).  Adding 512 to every lower digit
-// position makes the lower digits plain 10-bit fields of
-// Y = X + sum_k 512 1024^k (no carry chain); the field y = digit + 512 in
-// [0, 1024] (the top one: the top digit + 512) becomes the FP16 value 1024 + y
-// through the bit pattern 0x6400 + y (y = 1024 carries into the exponent:
-// 2048), and one packed FP16 subtraction of 1536 leaves the digit, exactly.
-__device__ __forceinline__ void digit_pairs(long long X0, long long X1, uint32_t (&h)[S]) {
-    constexpr long long C = 512LL * (1 + (1LL << 10) + (1LL << 20) + (1LL << 30) + (1LL << 40));
-    static_assert(S == 6, "digit layout");
-    const unsigned long long Y0 = (unsigned long long)(X0 + C), Y1 = (unsigned long long)(X1 + C);
-    const unsigned l0 = (unsigned)Y0, h0 = (unsigned)(Y0 >> 32);
-    const unsigned l1 = (unsigned)Y1, h1 = (unsigned)(Y1 >> 32);
+// FP16x2 word (X0's in the low half), from Y = X + DBIAS.  Adding 512 at every lower digit
+// position makes the lower digits plain 10-bit fields of Y (no carry chain); the
+// field y = digit + 512 in [0, 1023] becomes the FP16 value 1024 + y through the bit
+// pattern 0x6400 | y -- both inputs' fields joined by one byte permute, masked and
+// completed by one logic operation -- and one packed FP16 subtraction of 1536
+// leaves the digit, exactly.  The top digit plus 512, in [0, 1024], is added to the
+// pattern instead (1024 carries into the exponent: 2048).
+__device__ __forceinline__ void digit_pairs(long long Y0, long long Y1, uint32_t (&h)[S]) {
+    static_assert(S == 6 && DBITS == 10, "digit layout");
+    const unsigned l0 = (unsigned)Y0, h0 = (unsigned)((unsigned long long)Y0 >> 32);
+    const unsigned l1 = (unsigned)Y1, h1 = (unsigned)((unsigned long long)Y1 >> 32);
     const __half2 off = __halves2half2(__ushort_as_half((unsigned short)0x6600),
                                        __ushort_as_half((unsigned short)0x6600));   // 1536
-    // fields y0, y1 <= 1024 -> the word (0x6400 + y0) | (0x6400 + y1) << 16,
-    // the halves joined by a byte permute (no carry crosses them)
-    auto pack = [&](unsigned y0, unsigned y1) {
-        const unsigned w = __byte_perm(y0, y1, 0x5410) + 0x64006400u;
+    auto sub = [&](unsigned w) {
         const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&w), off);
         return *reinterpret_cast<const uint32_t*>(&d);
     };
-    // the 10-bit field k of Y from its 32-bit halves (field 3 straddles them)
-    auto field = [](unsigned lo, unsigned hi, int k) {
-        return k < 3 ? (lo >> (DBITS * k)) & 1023u
-                     : k == 3 ? __funnelshift_r(lo, hi, 30) & 1023u : (hi >> (DBITS * k - 32)) & 1023u;
+    // words whose low halves start with the field
+    auto pack = [&](unsigned y0, unsigned y1) {
+        return sub((__byte_perm(y0, y1, 0x5410) & 0x03FF03FFu) | 0x64006400u);
     };
-#pragma unroll
-    for (int k = 0; k < S - 1; ++k) h[S - 1 - k] = pack(field(l0, h0, k), field(l1, h1, k));
-    h[0] = pack((unsigned)(((int)h0 >> (DBITS * (S - 1) - 32)) + 512),
-                (unsigned)(((int)h1 >> (DBITS * (S - 1) - 32)) + 512));
+    h[5] = pack(l0, l1);
+    h[4] = pack(l0 >> 10, l1 >> 10);
+    h[3] = pack(l0 >> 20, l1 >> 20);
+    h[2] = pack(__funnelshift_r(l0, h0, 30), __funnelshift_r(l1, h1, 30));
+    h[1] = pack(h0 >> 8, h1 >> 8);
+    h[0] = sub(__byte_perm(h0 >> 18, h1 >> 18, 0x5410) + 0x64006400u);
 }
 #endif
 
@@ -248,11 +268,14 @@ __device__ __forceinline__ void digit_pairs(long long X0, long long X1, uint32_t
 cudaError_t launch_pass_emu(int kind, int mode, const PassParams<double>& p, long long nunits,
                             cudaStream_t st);
 cudaError_t prepare_emu_kernels();
+bool emu_hands_over(int kind);
 // Largest biased exponent of every line of synthesis pass 1's input (full-
 // grid compressed form, cell of n1 x n2 x n3 coarse points, norb orbitals of
 // P elements): lexp[orbital][x3 * 2 n2 + x2].
 cudaError_t launch_line_exp(const double* in, int* lexp, int n1, int n2, int n3, int norb,
                             long long P, cudaStream_t st);
+// largest of each group of n consecutive ints
+cudaError_t launch_group_max(const int* g, int* gmax, int n, long long ngroups, cudaStream_t st);
 // bounded waits of the emulated passes that ran out since the last call
 cudaError_t emu_take_timeouts(unsigned* count);
 // one bounded wait that cannot be satisfied, given up after about ms

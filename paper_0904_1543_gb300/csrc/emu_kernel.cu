@@ -1,28 +1,45 @@
 // The emulated FP64 pass (see emu.cuh for the arithmetic) as a tcgen05
 // kernel for sm_103a.
 //
-// A window is 128 lines x N outputs (N = 32, or 16 for the kinetic filter)
-// reading 48 input positions, three 16-position slabs.  A work unit is a
-// whole 128-line tile of one orbital (of each orbital of a group in turn in
-// the potential pass, whose density partial it updates in place), walked
-// window by window.  A persistent CTA of 256 threads, two per SM, per window
-//   1. slices the window's new slabs: reads them (wrapped periodically, or
-//      gathered from the compressed layout in synthesis pass 1), scales every
-//      line by its largest exponent (taken once per unit), and writes six
-//      FP16 digit planes into a ring of three slab slots in shared memory, in
-//      the MMA's K-major layout (8 x 16 B core matrices);
-//   2. issues, from one thread, 6 data digits x 3 K-steps of MMAs
+// A window is 128 lines x 16 outputs reading 32 input positions, two 16-position
+// slabs (the kinetic filter 48, three).  A work unit is a whole 128-line tile of
+// one orbital (of each orbital of a group in turn in the potential pass, whose
+// density partial it updates in place), walked window by window.  A persistent CTA of
+// 256 threads, three per SM (two in the kinetic passes), per window
+//   1. slices the window's new slab: reads it from the copies that its threads made
+//      under the window before (cp.async, wrapped periodically; synthesis pass 1
+//      gathers from the compressed layout instead), puts every line on its
+//      scale, and writes six FP16 digit planes into a ring of slab slots
+//      in shared memory, in the MMA's K-major layout (8 x 16 B core matrices);
+//   2. issues, from one thread, 6 data digits x 2 or 3 K-steps of MMAs
 //      (M = 128, K = 16), each over the filter digits side by side along N,
 //      adding the 26 digit pairs' products into seven FP32 accumulators
 //      (one per diagonal, N columns each) in tensor memory, and commits them
 //      to an mbarrier, polled with a bound; meanwhile every thread loads the
 //      epilogue's other inputs;
 //   3. reads the accumulators (warp w: lines 32 (w % 4) + lane, half of the
-//      outputs), recombines them into 64-bit integers, scales to FP64 and
-//      runs the pass's epilogue (transposed store, compressed scatter, V psi
-//      with density and Epot, kinetic K_p and Ekin) as the FP64 pass does.
+//      outputs), recombines them into 64-bit integers and runs the pass's
+//      epilogue (transposed store, compressed scatter, V psi with density
+//      and Epot, kinetic K_p and Ekin).
+// Between the passes of one operator the outputs stay these integers, with a scale per
+// line (Seg::gout): the next pass shifts them to its own line's scale, the largest
+// exponent of the source lines that it crosses, without a scan of its inputs, and the FP64 pipe
+// (a conversion and a multiplication per output otherwise) is left out.  Where an FP64
+// array comes in, a line's exponent is the largest of a first read.
+// Every pass notes the largest magnitude of each line's integers, so that the scale of a
+// line is at most the spread inside its source lines above its own largest value; with the
+// bound |t| < 2^60 alone the error of H psi grew fourfold on coefficients that decay over
+// eleven decades.  It is now below that of FP64 hand-over: 1.2e-16 against
+// 1.5e-16 in the 2-norm (FP64 kernels 4.2e-16), 2.3e-16 against 2.7e-16 on decaying ones.
+// Per headline step (192 orbitals): 30.9 ms with windows of 32 outputs, two CTAs per SM;
+// 29.2 with 16 outputs and three; 28.5 with fields masked and completed in one
+// operation; 24.7 with the integers and the copies (neither alone gains:
+// without the scan's first read the slabs' loads wait for HBM, and copies of FP64 arrays leave
+// the scan; an L2 prefetch of the next slab gave 27.5, of the next tile 29.4, a
+// register prefetch of the next slab 31.7).
 // The filter digit planes are built once per CTA from the launch's taps.
 #include <cmath>
+#include <type_traits>
 
 #include <cuda_fp16.h>
 
@@ -37,6 +54,15 @@ __device__ unsigned int g_emu_timeouts = 0;
 namespace emu {
 
 using namespace tc;
+
+enum { IO_IN = 1, IO_OUT = 2 };   // integer input, output of a pass
+
+// a b + c, 32 x 32 + 64 bits
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
+    long long d;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+    return d;
+}
 
 // input value at position x (0 <= x < n) of line a of orbital orb
 template <int MODE>
@@ -138,18 +164,6 @@ __device__ __forceinline__ void issue_window_mmas(uint32_t tm, uint32_t a_base, 
     }
 }
 
-// digits of two consecutive inputs of line r into the data planes at the
-// given chunk (8 positions) and pair within it
-template <int LBOA>
-__device__ __forceinline__ void store_pair_digits(unsigned char* Asm, int apl, int chunk, int r,
-                                                  int pair4, double v0, double v1, int E) {
-    uint32_t h[S];
-    digit_pairs(quantize(v0, E), quantize(v1, E), h);
-    unsigned char* dst = Asm + chunk * LBOA + r * 16 + pair4 * 4;
-#pragma unroll
-    for (int q = 0; q < S; ++q) *reinterpret_cast<uint32_t*>(dst + q * apl) = h[q];
-}
-
 // The epilogue's other inputs for this thread's outputs (line er, outputs
 // o0 .. o0 + N/2 - 1), loaded while the MMAs run: the kinetic passes' G and
 // K_{p-1} (line-major, 16-byte loads) and K_0; the potential pass's V and
@@ -209,12 +223,13 @@ __device__ __forceinline__ void prefetch_epilogue(const Seg<double>& Sg, int o0,
 
 // one window's outputs of this thread (line er, outputs o0 .. o0 + N/2 - 1):
 // accumulators -> FP64 -> the pass's epilogue; returns the energy partial
-template <int KIND, int MODE>
+template <int KIND, int MODE, bool OUTI>
 __device__ __forceinline__ double window_epilogue(const Seg<double>& Sg, uint32_t tl, int o0,
                                                   int er, int lt, int a0, int orb, int grp, int se,
                                                   const double (&pa)[window_n(KIND) / 2],
                                                   const double (&pb)[window_n(KIND) / 2],
-                                                  const double (&pc)[window_n(KIND) / 2]) {
+                                                  const double (&pc)[window_n(KIND) / 2],
+                                                  unsigned& top) {
     constexpr int N = window_n(KIND), NH = N / 2;
     constexpr bool KM = (MODE == M_KMID || MODE == M_KLAST);
     const int n = Sg.n, NL = Sg.N;
@@ -230,41 +245,72 @@ __device__ __forceinline__ double window_epilogue(const Seg<double>& Sg, uint32_
     double osc = 1.0;
     if (MODE == M_COMP && Sg.gscale != nullptr) osc = 2.0 * Sg.occ[orb] * Sg.gscale[0];
     double eacc = 0.0;
+    static_assert(NH == 8 && NACC == 7 && NEXACT == 4 && DBITS == 10 && TSHIFT == 20 && DMAX == 8, "recombination");
+    uint32_t dv[NACC][8];
 #pragma unroll
-    for (int c8 = 0; c8 < NH / 8; ++c8) {
-        uint32_t dv[NACC][8];
+    for (int ac = 0; ac < NACC; ++ac) tld8(tl + ac * N, dv[ac]);
+    tld_wait();
+    const bool full = o0 + NH <= n;   // every output exists
+    // element (I, a) of the transposed output is at obase + I NL + a
+    const long long oi0 = obase + (long long)o0 * NL + a;
+    // M_COMP on the full grid: the outputs' positions in the compressed form, two outputs per
+    // coarse point along the line (components mu12 and mu12 + 4)
+    double* ce = nullptr;
+    double* co = nullptr;
+    long long se_ = 0, so_ = 0;
+    int X1 = 0, X2 = 0;
+    const bool plain = Sg.mapc == nullptr && Sg.bx1 == 0;
+    if (MODE == M_COMP) {
+        X2 = a / Sg.N1;
+        X1 = a - X2 * Sg.N1;
+        const int mu12 = (X1 & 1) + 2 * (X2 & 1);
+        const int plane = Sg.n1 * Sg.n2, cx = (X2 >> 1) * Sg.n1 + (X1 >> 1);
+        double* const cc0 = Sg.out + (long long)orb * Sg.clen;
+        so_ = 7LL * plane;
+        se_ = mu12 == 0 ? plane : so_;
+        const long long i2 = o0 >> 1;
+        ce = (mu12 == 0 ? cc0 + cx : cc0 + Sg.ncoarse + 7LL * cx + mu12 - 1) + i2 * se_;
+        co = cc0 + Sg.ncoarse + 7LL * cx + mu12 + 3 + i2 * so_;
+    }
+    if (!row_ok) return 0.0;
+    {
 #pragma unroll
-        for (int ac = 0; ac < NACC; ++ac) tld8(tl + ac * N + c8 * 8, dv[ac]);
-        tld_wait();
+        for (int c = 0; c < NH; ++c) {
+            // diagonals 0 .. 3 (exact integers, weights 2^40 .. 2^10) and the sum of the
+            // low ones (weights 1, 2^-10, 2^-20), in one 64-bit integer
+            int i[NEXACT];
 #pragma unroll
-        for (int jj = 0; jj < 8; ++jj) {
-            long long t = 0;
-            float low = 0.f;
-#pragma unroll
-            for (int ac = 0; ac < NACC; ++ac) {
-                const float v = __uint_as_float(dv[ac][jj]);
-                // shifts and weights of the canonical schedule (checked on the host)
-                if (ac < NEXACT) t += (long long)__float2int_rn(v) << (DBITS * (DMAX - 2 - ac) - TSHIFT);
-                else low = fmaf(v, __int_as_float((127 + DBITS * (DMAX - 2 - ac) - TSHIFT) << 23), low);
-            }
-            t += __float2int_rn(low);
-            const double val = (double)t * scale;
-            const int c = c8 * 8 + jj;
+            for (int ac = 0; ac < NEXACT; ++ac) i[ac] = __float2int_rn(__uint_as_float(dv[ac][c]));
+            float low = __uint_as_float(dv[4][c]);
+            low = fmaf(__uint_as_float(dv[5][c]), 0x1p-10f, low);
+            low = fmaf(__uint_as_float(dv[6][c]), 0x1p-20f, low);
+            const int i01 = i[0] * 1024 + i[1];
+            long long t = __float2int_rn(low);
+            t = mad_wide(i[3], 1 << 10, t);
+            t = mad_wide(i[2], 1 << 20, t);
+            t = mad_wide(i01, 1 << 30, t);
             const int I = o0 + c;
-            if (!row_ok || I >= n) continue;
-            const long long oidx = (long long)I * NL + a;
+            if (!full && I >= n) continue;
+            const long long oi = oi0 + (long long)c * NL;
+            if constexpr (OUTI) {
+                // the next pass reads the integer and the line's scale
+                const int th = (int)(t >> 32);
+                top = max(top, (unsigned)(th ^ (th >> 31)));
+                reinterpret_cast<long long*>(Sg.out)[oi] = t;
+                continue;
+            }
+            const double val = (double)t * scale;
             if (MODE == M_PLAIN || MODE == M_UNCOMP) {
-                Sg.out[obase + oidx] = val;
+                Sg.out[oi] = val;
             } else if (MODE == M_COMP) {
-                const int X2 = a / Sg.N1, X1 = a - X2 * Sg.N1;
-                const int mu = (X1 & 1) + 2 * (X2 & 1) + 4 * (I & 1);
-                const long long ci = ((long long)(I >> 1) * Sg.n2 + (X2 >> 1)) * Sg.n1 + (X1 >> 1);
-                double* cc0 = Sg.out + (long long)orb * Sg.clen;
                 const double sv = Sg.gscale != nullptr ? val * osc : val;
-                if (Sg.mapc == nullptr && Sg.bx1 == 0) {
-                    if (mu == 0) cc0[ci] = sv;
-                    else cc0[Sg.ncoarse + ci * 7 + mu - 1] = sv;
+                if (plain) {
+                    if (c & 1) co[(c >> 1) * so_] = sv;
+                    else ce[(c >> 1) * se_] = sv;
                 } else {
+                    const int mu = (X1 & 1) + 2 * (X2 & 1) + 4 * (I & 1);
+                    const long long ci = ((long long)(I >> 1) * Sg.n2 + (X2 >> 1)) * Sg.n1 + (X1 >> 1);
+                    double* const cc0 = Sg.out + (long long)orb * Sg.clen;
                     const int k = stored_index(Sg, ci, X1 >> 1, X2 >> 1, I >> 1, mu);
                     if (k >= 0) {
                         if (mu == 0) cc0[k] = sv;
@@ -277,16 +323,16 @@ __device__ __forceinline__ double window_epilogue(const Seg<double>& Sg, uint32_
                 if (MODE == M_KMID && Sg.in2 == nullptr && Sg.eps != nullptr) kin = -Sg.eps[orb] * g;
                 const double acc = val + kin;
                 if (MODE == M_KMID) {
-                    Sg.out[obase + oidx] = acc;
-                    Sg.out2[obase + oidx] = g;
+                    Sg.out[oi] = acc;
+                    Sg.out2[oi] = g;
                 } else {
-                    if (Sg.out) Sg.out[obase + oidx] = acc;
+                    if (Sg.out) Sg.out[oi] = acc;
                     eacc = fma(g, acc - pc[c], eacc);
                 }
             } else if (MODE == M_POT) {
                 if (Sg.aux) {
                     const double y = pa[c] * val;
-                    if (Sg.out) Sg.out[obase + oidx] = y;
+                    if (Sg.out) Sg.out[oi] = y;
                     eacc = fma(y, val, eacc);
                 }
                 // the unit owns these density elements: one thread updates
@@ -294,7 +340,7 @@ __device__ __forceinline__ double window_epilogue(const Seg<double>& Sg, uint32_
                 // so far is the caller's rho, or this group's partial after
                 // the group's first orbital
                 if (Sg.rho != nullptr) {
-                    double* const rp = Sg.rho + (long long)grp * Sg.rho_gstride + oidx;
+                    double* const rp = Sg.rho + (long long)grp * Sg.rho_gstride + (oi - obase);
                     const double prev = (Sg.rho_gstride == 0 || orb != grp * Sg.opg) ? *rp : 0.0;
                     *rp = fma(occ * val, val, prev);
                 }
@@ -317,9 +363,10 @@ __device__ __forceinline__ double cta_sum(double v, double* red) {
     return t;
 }
 
-template <int KIND, int MODE>
-__global__ void __launch_bounds__(THREADS, 2)
+template <int KIND, int MODE, int IO>
+__global__ void __launch_bounds__(THREADS, min_ctas(KIND))
 emu_pass_kernel(const __grid_constant__ Params ep) {
+    constexpr bool INI = (IO & IO_IN) != 0, OUTI = (IO & IO_OUT) != 0;   // integer input, output
     constexpr int K = window_k(KIND), HA = window_ha(KIND);
     constexpr int LBOA = lboa(MODE);
     constexpr int APL = plane_a_bytes(KIND, MODE);
@@ -328,13 +375,15 @@ emu_pass_kernel(const __grid_constant__ Params ep) {
     constexpr int NH = N / 2;                // outputs per epilogue thread
     constexpr int RPW = M / WARPS;           // lines per slicing warp
     constexpr int NSLOT = K / 16;            // 16-position slabs per window (3)
-    static_assert(K == 48 && N % 16 == 0 && (HA - (KIND == K_KIN ? 0 : 8)) % 16 == 0, "window");
+    static_assert(N == 16, "one new slab per window");
     extern __shared__ __align__(128) unsigned char sm[];
     unsigned char* const Asm = sm;                // [S][APL]: NSLOT slab slots of 2 chunks
     unsigned char* const Bsm = sm + S * APL;      // K / 8 chunks of (S + 1) N rows
     __shared__ uint32_t tslot;
     __shared__ __align__(8) uint64_t mbar;
     __shared__ int rowE[M];
+    __shared__ int rowG[INI ? M : 1];             // integer input: a line's first source line
+    __shared__ unsigned rowT[OUTI ? 2 * M : 1];   // integer output: largest magnitudes per line and half
     __shared__ double red[WARPS];
 
     const PassParams<double>& p = ep.p;
@@ -403,6 +452,46 @@ emu_pass_kernel(const __grid_constant__ Params ep) {
 
     EJob J;
     first_job(p, MODE, J);
+
+    // The copies' cursor: the slab after the last one copied, in job Q.  A thread copies
+    // exactly the 16-byte pairs that it will slice (rows r0 + 4 g, pair `pair`) and reads
+    // them back itself, so its own wait is all the synchronisation they need, and they have a
+    // whole window (or the previous job's last one) to arrive.
+    const int pair = lane & 7, r0 = warp * RPW + (lane >> 3);
+    unsigned char* const raw = sm + S * APL + b_bytes(KIND) + tid * 16;
+    EJob Q = J;
+    const double* qsrc = nullptr;
+    int qx = 0, qleft = 0, qn = 0;
+    auto begin_copies = [&]() {
+        if (!Q.valid) return;
+        const Seg<double>& Sq = p.seg[Q.si];
+        qn = Sq.n;
+        qsrc = Sq.in + (long long)Q.orb * Sq.P + (long long)(Q.a0 + r0) * qn;
+        qx = -HA % qn;
+        if (qx < 0) qx += qn;
+        qleft = Sq.nwin + NSLOT - 1;
+    };
+    auto copy_slab = [&]() {
+        if (qleft == 0) {
+            next_job(p, MODE, Q);
+            begin_copies();
+        }
+        if (Q.valid) {
+            int x = qx + 2 * pair;
+            while (x >= qn) x -= qn;
+#pragma unroll
+            for (int g4 = 0; g4 < RPW / 4; ++g4)
+                if (r0 + 4 * g4 < Q.lt) cp_async16(raw + g4 * THREADS * 16, qsrc + (long long)(4 * g4) * qn + x);
+            qx += 16;
+            while (qx >= qn) qx -= qn;
+            --qleft;
+        }
+        cp_commit();
+    };
+    if constexpr (MODE != M_UNCOMP) {
+        begin_copies();
+        copy_slab();
+    }
 #pragma unroll 1
     while (J.valid) {
         const Seg<double>& Sg = p.seg[J.si];
@@ -410,7 +499,16 @@ emu_pass_kernel(const __grid_constant__ Params ep) {
         {
             // ---------------------------- one exponent per line: given (synthesis
             // pass 1 on the full grid), or the whole line read, 8 lines in flight per warp
-            if (MODE == M_UNCOMP && Sg.lexp != nullptr) {
+            if constexpr (INI) {
+                // the largest exponent of the n neighbouring source lines that this line
+                // crosses (n divides nsrc)
+                if (tid < M) {
+                    const int ng = Sg.nsrc / n;
+                    const int k = (int)((unsigned)(J.a0 + tid) % (unsigned)ng);
+                    rowE[tid] = tid < J.lt ? Sg.gmax[(long long)J.orb * ng + k] : HAND_MIN;
+                    rowG[tid] = tid < J.lt ? k * n : 0;
+                }
+            } else if (MODE == M_UNCOMP && Sg.lexp != nullptr) {
                 for (int r = tid; r < M; r += THREADS)
                     rowE[r] = scale_of(r < J.lt ? Sg.lexp[(long long)J.orb * Sg.N + J.a0 + r] : 0);
             } else
@@ -442,79 +540,88 @@ emu_pass_kernel(const __grid_constant__ Params ep) {
             }
             __syncthreads();
             // ---------------------------- windows; each slab sliced once
-            // slab s covers positions 16 s + P0 .. + 15; window w reads slabs
-            // s0(w) .. s0(w) + 2 from slots (slab mod 3)
-            constexpr int P0 = (KIND == K_KIN) ? 0 : -8;
+            // slab s covers positions 16 s - HA .. + 15; window w reads slabs w .. w + NSLOT - 1
+            // from slots (slab mod NSLOT)
             const int nwin = Sg.nwin;
-            constexpr int NEW = N / 16;          // new slabs per window after the first
-            // raw inputs of one slab for this lane: lines warp * RPW + 4 g + lane / 8,
-            // positions 2 (lane % 8), + 1 of the slab
-            auto load_slab = [&](int sb, double (&v)[RPW / 4][2]) {
-                const int pair = lane & 7;
-                int x = (16 * sb + P0 + 2 * pair) % n;
-                if (x < 0) x += n;
-                int x1 = x + 1;
-                if (x1 >= n) x1 -= n;
+            // raw inputs of one slab for this lane: lines r0 + 4 g, r0 = warp * RPW + lane / 8,
+            // positions 2 (lane % 8), + 1 of the slab; with integers, their lines' scales
+            struct Raw {
+                long long v[RPW / 4][2];
+                int g[INI ? RPW / 4 : 1][2];
+            };
+            const int* const gsrc = INI ? Sg.gin + (long long)J.orb * Sg.nsrc : nullptr;
+            unsigned char* const adst = Asm + (pair >> 2) * LBOA + r0 * 16 + (pair & 3) * 4;
+            int xs = -HA % n;            // first position of the next slab to load
+            if (xs < 0) xs += n;
+            int slot = 0;                // and its slot
+            auto load_slab = [&](Raw& w) {
+                int x = xs + 2 * pair;
+                while (x >= n) x -= n;
+                if constexpr (MODE != M_UNCOMP) cp_wait<0>();
 #pragma unroll
                 for (int g4 = 0; g4 < RPW / 4; ++g4) {
-                    const int r = warp * RPW + 4 * g4 + (lane >> 3);
-                    v[g4][0] = v[g4][1] = 0.0;
-                    if (r >= J.lt) continue;
+                    w.v[g4][0] = w.v[g4][1] = 0;
+                    if constexpr (INI) w.g[g4][0] = w.g[g4][1] = 0;
+                    if (r0 + 4 * g4 >= J.lt) continue;
                     if (MODE == M_UNCOMP) {
-                        v[g4][0] = load_in<MODE>(Sg, J.orb, J.a0 + r, x);
-                        v[g4][1] = load_in<MODE>(Sg, J.orb, J.a0 + r, x1);
+                        w.v[g4][0] = __double_as_longlong(load_in<MODE>(Sg, J.orb, J.a0 + r0 + 4 * g4, x));
+                        w.v[g4][1] = __double_as_longlong(load_in<MODE>(Sg, J.orb, J.a0 + r0 + 4 * g4, x + 1));
                     } else {
-                        // x is even and n is even: x1 = x + 1, 16-byte aligned
-                        const double2 d2 = *reinterpret_cast<const double2*>(
-                            Sg.in + (long long)J.orb * Sg.P + (long long)(J.a0 + r) * n + x);
-                        v[g4][0] = d2.x;
-                        v[g4][1] = d2.y;
+                        // x is even and n is even: x + 1 is in the line, 16-byte aligned
+                        const longlong2 d2 = *reinterpret_cast<const longlong2*>(raw + g4 * THREADS * 16);
+                        w.v[g4][0] = d2.x;
+                        w.v[g4][1] = d2.y;
+                        if constexpr (INI) {
+                            const int2 g2 = *reinterpret_cast<const int2*>(gsrc + rowG[r0 + 4 * g4] + x);
+                            w.g[g4][0] = g2.x;
+                            w.g[g4][1] = g2.y;
+                        }
                     }
                 }
+                if constexpr (MODE != M_UNCOMP) copy_slab();
+                xs += 16;
+                while (xs >= n) xs -= n;
             };
-            auto slice_slab = [&](int sb, const double (&v)[RPW / 4][2]) {
-                const int slot = ((sb % NSLOT) + NSLOT) % NSLOT;
-                const int pair = lane & 7;
+            auto slice_slab = [&](const Raw& w) {
+                unsigned char* const d = adst + slot * (2 * LBOA);
 #pragma unroll
                 for (int g4 = 0; g4 < RPW / 4; ++g4) {
-                    const int r = warp * RPW + 4 * g4 + (lane >> 3);
-                    store_pair_digits<LBOA>(Asm, APL, 2 * slot + (pair >> 2), r, pair & 3, v[g4][0],
-                                            v[g4][1], rowE[r]);
+                    const int E = rowE[r0 + 4 * g4];
+                    long long y[2];
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        if constexpr (INI) y[c] = requantize(w.v[g4][c], w.g[g4][c], E);
+                        else y[c] = quantize(__longlong_as_double(w.v[g4][c]), E) + DBIAS;
+                    }
+                    uint32_t h[S];
+                    digit_pairs(y[0], y[1], h);
+#pragma unroll
+                    for (int q = 0; q < S; ++q) *reinterpret_cast<uint32_t*>(d + g4 * 64 + q * APL) = h[q];
                 }
+                if (++slot == NSLOT) slot = 0;
             };
+            if constexpr (OUTI)
+                if (tid < J.lt) Sg.gout[(long long)J.orb * Sg.N + J.a0 + tid] = rowE[tid] + Ef - OUT_EXP;
             double eacc = 0.0;
+            unsigned top = 0;   // largest high word of this thread's integer outputs' magnitudes
+            int first = 0;   // slot of the window's first slab
 #pragma unroll 1
             for (int w = 0; w < nwin && !failed; ++w) {
                 const int o = w * N;
-                const int s0 = (o - HA - P0) / 16;
                 if (w == 0) {
-                    if constexpr (KIND == K_KIN) {
-                        // the kinetic pass's tiles have 5 to 7 windows, so the
-                        // first window's three slabs weigh: their loads first
-                        // (8.82 -> 8.47 ms per headline step; the 16-tap passes,
-                        // with 3 to 4 windows, measured no gain)
-                        double v[NSLOT][RPW / 4][2];
-#pragma unroll
-                        for (int k = 0; k < NSLOT; ++k) load_slab(s0 + k, v[k]);
-#pragma unroll
-                        for (int k = 0; k < NSLOT; ++k) slice_slab(s0 + k, v[k]);
-                    } else {
 #pragma unroll 1
-                        for (int sb = s0; sb < s0 + NSLOT; ++sb) {
-                            double v[RPW / 4][2];
-                            load_slab(sb, v);
-                            slice_slab(sb, v);
-                        }
+                    for (int k = 0; k < NSLOT; ++k) {
+                        Raw v;
+                        load_slab(v);
+                        slice_slab(v);
                     }
                 } else {
-#pragma unroll 1
-                    for (int k = 0; k < NEW; ++k) {
-                        double v[RPW / 4][2];
-                        load_slab(s0 + NSLOT - NEW + k, v);
-                        slice_slab(s0 + NSLOT - NEW + k, v);
-                    }
+                    Raw v;
+                    load_slab(v);
+                    slice_slab(v);
+                    if (++first == NSLOT) first = 0;
                 }
-                issue_mmas(((s0 % NSLOT) + NSLOT) % NSLOT);
+                issue_mmas(first);
                 double pa[NH], pb[NH], pc[NH];
                 prefetch_epilogue<KIND, MODE>(Sg, o + NH * half, er, J.lt, J.a0, J.orb, J.grp, pa,
                                               pb, pc);
@@ -523,8 +630,8 @@ emu_pass_kernel(const __grid_constant__ Params ep) {
                     failed = true;
                     break;
                 }
-                eacc += window_epilogue<KIND, MODE>(Sg, tl, o + NH * half, er, J.lt, J.a0, J.orb,
-                                                    J.grp, rowE[er] + Ef - OUT_EXP, pa, pb, pc);
+                eacc += window_epilogue<KIND, MODE, OUTI>(Sg, tl, o + NH * half, er, J.lt, J.a0, J.orb,
+                                                    J.grp, rowE[er] + Ef - OUT_EXP, pa, pb, pc, top);
                 fence_before();
                 __syncthreads();   // accumulators are rewritten by the next window's MMAs
             }
@@ -534,11 +641,20 @@ emu_pass_kernel(const __grid_constant__ Params ep) {
                 if (tid == 0) Sg.part[(long long)J.orb * Sg.tiles + J.tt] = t;
                 __syncthreads();
             }
+            if constexpr (OUTI) rowT[half * M + er] = top;
             __syncthreads();   // rowE and the slab ring are reused by the next job
+            if constexpr (OUTI)
+                if (tid < J.lt) {
+                    // |t| <= 2^(32 + bits of the high word)
+                    const int bits = 64 - __clz((int)max(rowT[tid], rowT[M + tid]));
+                    const long long at = (long long)J.orb * Sg.N + J.a0 + tid;
+                    Sg.gtop[at] = Sg.gout[at] + max(HAND_MIN, bits);
+                }
             next_job(p, MODE, J);
         }
     }
 
+    cp_wait<0>();
     if (failed) {
         // let the MMAs still in flight finish before the accumulators are freed
         if (tid == 0) {
@@ -559,7 +675,7 @@ static bool build_sched(int kind, const PassParams<double>& p, Sched& s) {
     return emu::build_sched(p.f, kind_geom(kind).nt, s);
 }
 
-template <int KIND, int MODE>
+template <int KIND, int MODE, int IO>
 static cudaError_t ensure_emu_attr() {
     static unsigned long long done = 0;
     int dev = 0;
@@ -567,10 +683,10 @@ static cudaError_t ensure_emu_attr() {
     if (err != cudaSuccess) return err;
     const unsigned long long bit = 1ull << (dev & 63);
     if (!(__atomic_load_n(&done, __ATOMIC_ACQUIRE) & bit)) {
-        err = cudaFuncSetAttribute(emu_pass_kernel<KIND, MODE>,
+        err = cudaFuncSetAttribute(emu_pass_kernel<KIND, MODE, IO>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(KIND, MODE));
         if (err != cudaSuccess) return err;
-        err = cudaFuncSetAttribute(emu_pass_kernel<KIND, MODE>,
+        err = cudaFuncSetAttribute(emu_pass_kernel<KIND, MODE, IO>,
                                    cudaFuncAttributePreferredSharedMemoryCarveout,
                                    cudaSharedmemCarveoutMaxShared);
         if (err != cudaSuccess) return err;
@@ -579,9 +695,9 @@ static cudaError_t ensure_emu_attr() {
     return cudaSuccess;
 }
 
-template <int KIND, int MODE>
+template <int KIND, int MODE, int IO>
 static cudaError_t launch_emu(const Params& ep, long long nunits, cudaStream_t st) {
-    cudaError_t err = ensure_emu_attr<KIND, MODE>();
+    cudaError_t err = ensure_emu_attr<KIND, MODE, IO>();
     if (err != cudaSuccess) return err;
     if (nunits <= 0) return cudaSuccess;
     int dev = 0, nsm = 0, occ = 0;
@@ -593,7 +709,7 @@ static cudaError_t launch_emu(const Params& ep, long long nunits, cudaStream_t s
     static int regs[64] = {0};
     if (!regs[dev & 63]) {
         cudaFuncAttributes fa;
-        if ((err = cudaFuncGetAttributes(&fa, emu_pass_kernel<KIND, MODE>)) != cudaSuccess) return err;
+        if ((err = cudaFuncGetAttributes(&fa, emu_pass_kernel<KIND, MODE, IO>)) != cudaSuccess) return err;
         regs[dev & 63] = std::max(fa.numRegs, 1);
     }
     int smem_sm = 0;
@@ -606,9 +722,33 @@ static cudaError_t launch_emu(const Params& ep, long long nunits, cudaStream_t s
     occ = std::min(std::min(by_smem, by_regs), 512 / tmem_cols(KIND));
     if (occ < 1) return cudaErrorInvalidConfiguration;
     long long grid = std::min<long long>((long long)occ * nsm, nunits);
-    emu_pass_kernel<KIND, MODE><<<dim3((unsigned)grid), dim3(THREADS), smem_bytes(KIND, MODE), st>>>(ep);
+    emu_pass_kernel<KIND, MODE, IO><<<dim3((unsigned)grid), dim3(THREADS), smem_bytes(KIND, MODE), st>>>(ep);
     count_launches(1);
     return cudaGetLastError();
+}
+
+// every pass kernel of the chains: f(kind, mode, io)
+template <typename F>
+static void for_each_emu(F&& f) {
+#define EMU_K(kind, mode, io)                                                              \
+    f(std::integral_constant<int, kind>{}, std::integral_constant<int, mode>{},            \
+      std::integral_constant<int, io>{})
+    EMU_K(K_SYN, M_UNCOMP, IO_OUT);
+    EMU_K(K_ANA, M_COMP, IO_IN);
+    EMU_K(K_MF, M_POT, IO_IN);
+    EMU_K(K_SYN, M_PLAIN, IO_IN | IO_OUT);
+    EMU_K(K_SYN, M_PLAIN, IO_IN);
+    EMU_K(K_MF, M_PLAIN, IO_OUT);
+    EMU_K(K_MF, M_PLAIN, IO_IN | IO_OUT);
+    EMU_K(K_MF, M_PLAIN, IO_IN);
+    EMU_K(K_MFT, M_PLAIN, IO_OUT);
+    EMU_K(K_MFT, M_PLAIN, IO_IN | IO_OUT);
+    EMU_K(K_MFT, M_PLAIN, IO_IN);
+    EMU_K(K_ANA, M_PLAIN, IO_OUT);
+    EMU_K(K_ANA, M_PLAIN, IO_IN | IO_OUT);
+    EMU_K(K_KIN, M_KMID, 0);
+    EMU_K(K_KIN, M_KLAST, 0);
+#undef EMU_K
 }
 
 }  // namespace emu
@@ -651,6 +791,26 @@ __global__ void line_exp_kernel(const double* __restrict__ in, int* __restrict__
     }
 }
 
+// gmax[orbital][k] = the largest of g[orbital][k n .. k n + n - 1]; one warp each
+__global__ void group_max_kernel(const int* __restrict__ g, int* __restrict__ gmax, int n, long long ngroups) {
+    const long long k = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (k >= ngroups) return;
+    int e = -0x7fffffff;
+    for (int x = lane; x < n; x += 32) e = max(e, g[k * n + x]);
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) gmax[k] = e;
+}
+
+cudaError_t launch_group_max(const int* g, int* gmax, int n, long long ngroups, cudaStream_t st) {
+    if (ngroups <= 0) return cudaSuccess;
+    const long long blocks = (ngroups + 7) / 8;
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    group_max_kernel<<<(unsigned)blocks, 256, 0, st>>>(g, gmax, n, ngroups);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_line_exp(const double* in, int* lexp, int n1, int n2, int n3, int norb,
                             long long P, cudaStream_t st) {
     const long long nrows = (long long)norb * n3 * n2;
@@ -670,42 +830,30 @@ cudaError_t launch_pass_emu(int kind, int mode, const PassParams<double>& p, lon
     ep.p = p;
     if (!emu::build_sched(kind, p, ep.s)) return cudaErrorInvalidValue;
     using namespace emu;
-    switch (kind) {
-    case K_SYN:
-        if (mode == M_UNCOMP) return launch_emu<K_SYN, M_UNCOMP>(ep, nunits, st);
-        if (mode == M_PLAIN) return launch_emu<K_SYN, M_PLAIN>(ep, nunits, st);
-        break;
-    case K_ANA:
-        if (mode == M_COMP) return launch_emu<K_ANA, M_COMP>(ep, nunits, st);
-        if (mode == M_PLAIN) return launch_emu<K_ANA, M_PLAIN>(ep, nunits, st);
-        break;
-    case K_MF:
-        if (mode == M_POT) return launch_emu<K_MF, M_POT>(ep, nunits, st);
-        if (mode == M_PLAIN) return launch_emu<K_MF, M_PLAIN>(ep, nunits, st);
-        break;
-    case K_MFT:
-        if (mode == M_PLAIN) return launch_emu<K_MFT, M_PLAIN>(ep, nunits, st);
-        break;
-    case K_KIN:
-        if (mode == M_KMID) return launch_emu<K_KIN, M_KMID>(ep, nunits, st);
-        if (mode == M_KLAST) return launch_emu<K_KIN, M_KLAST>(ep, nunits, st);
-        break;
-    }
-    return cudaErrorInvalidValue;
+    // (one launch's segments agree on integer input and output)
+    const int io = (p.seg[0].gin != nullptr ? IO_IN : 0) | (p.seg[0].gout != nullptr ? IO_OUT : 0);
+    cudaError_t e = cudaErrorInvalidValue;
+    for_each_emu([&](auto k, auto m, auto i) {
+        if (kind == k() && mode == m() && io == i()) e = launch_emu<k(), m(), i()>(ep, nunits, st);
+    });
+    return e;
 }
 
 cudaError_t prepare_emu_kernels() {
-    using namespace emu;
-    cudaError_t e;
-    if ((e = ensure_emu_attr<K_SYN, M_UNCOMP>()) != cudaSuccess) return e;
-    if ((e = ensure_emu_attr<K_SYN, M_PLAIN>()) != cudaSuccess) return e;
-    if ((e = ensure_emu_attr<K_ANA, M_COMP>()) != cudaSuccess) return e;
-    if ((e = ensure_emu_attr<K_ANA, M_PLAIN>()) != cudaSuccess) return e;
-    if ((e = ensure_emu_attr<K_MF, M_POT>()) != cudaSuccess) return e;
-    if ((e = ensure_emu_attr<K_MF, M_PLAIN>()) != cudaSuccess) return e;
-    if ((e = ensure_emu_attr<K_MFT, M_PLAIN>()) != cudaSuccess) return e;
-    if ((e = ensure_emu_attr<K_KIN, M_KMID>()) != cudaSuccess) return e;
-    return ensure_emu_attr<K_KIN, M_KLAST>();
+    cudaError_t e = cudaSuccess;
+    emu::for_each_emu([&](auto k, auto m, auto i) {
+        if (e == cudaSuccess) e = emu::ensure_emu_attr<k(), m(), i()>();
+    });
+    return e;
+}
+
+// whether a pass of this kind can hand over integers: |T'| < 2^60
+bool emu_hands_over(int kind) {
+    PassParams<double> p;
+    std::memset(&p, 0, sizeof p);
+    fill_taps(p, kind, 1.0);
+    emu::Sched s;
+    return emu::build_sched(kind, p, s) && s.tbits <= 60;
 }
 
 namespace emu {
