@@ -80,9 +80,14 @@ __host__ __device__ constexpr int plane_a_bytes(int kind, int mode) { return win
 __host__ __device__ constexpr int b_bytes(int kind) { return window_k(kind) / 8 * lbo_b(kind); }
 // raw inputs of the next slab, 16 bytes x 4 rows per thread (not synthesis pass 1, which
 // gathers its inputs)
-__host__ __device__ constexpr int raw_bytes(int mode) { return mode == M_UNCOMP ? 0 : 4 * THREADS * 16; }
+// (kinetic passes: whole rows of 16 positions at a stride of RAWROW bytes, which eight
+// lanes read a row each without bank conflicts)
+constexpr int RAWROW = 16 * 8 + 16;
+__host__ __device__ constexpr int raw_bytes(int kind, int mode) {
+    return mode == M_UNCOMP ? 0 : kind == K_KIN ? M * RAWROW : 4 * THREADS * 16;
+}
 __host__ __device__ constexpr int smem_bytes(int kind, int mode) {
-    return S * plane_a_bytes(kind, mode) + b_bytes(kind) + raw_bytes(mode);
+    return S * plane_a_bytes(kind, mode) + b_bytes(kind) + raw_bytes(kind, mode);
 }
 
 // Schedule of one launch: which (filter digit p, data digit q) pairs go to

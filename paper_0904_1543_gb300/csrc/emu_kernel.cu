@@ -165,9 +165,8 @@ __device__ __forceinline__ void issue_window_mmas(uint32_t tm, uint32_t a_base, 
 }
 
 // The epilogue's other inputs for this thread's outputs (line er, outputs
-// o0 .. o0 + N/2 - 1), loaded while the MMAs run: the kinetic passes' G and
-// K_{p-1} (line-major, 16-byte loads) and K_0; the potential pass's V and
-// the density accumulated so far.
+// o0 .. o0 + N/2 - 1), loaded while the MMAs run: the kinetic passes' K_{p-1}
+// (line-major, 16-byte loads) and K_0; the potential pass's V.
 template <int KIND, int MODE>
 __device__ __forceinline__ void prefetch_epilogue(const Seg<double>& Sg, int o0, int er, int lt,
                                                   int a0, int orb, int grp,
@@ -182,30 +181,26 @@ __device__ __forceinline__ void prefetch_epilogue(const Seg<double>& Sg, int o0,
     const long long obase = (long long)orb * Sg.P;
     const bool full = er < lt && o0 + NH <= n;   // all outputs exist: vector loads
 #pragma unroll
-    for (int c = 0; c < NH; ++c) pa[c] = pb[c] = pc[c] = 0.0;
+    for (int c = 0; c < NH; ++c) {
+        if (!KM) pa[c] = 0.0;   // (the kinetic passes' G is there already)
+        pb[c] = pc[c] = 0.0;
+    }
     if (er >= lt) return;
     if (KM) {
-        const double* gi = Sg.in + obase + (long long)a * n + o0;
         const double* ki = Sg.in2 ? Sg.in2 + obase + (long long)a * n + o0 : nullptr;
-        if (full) {
+        if (ki != nullptr) {
+            if (full) {
 #pragma unroll
-            for (int c = 0; c < NH; c += 2) {
-                const double2 g2 = *reinterpret_cast<const double2*>(gi + c);
-                pa[c] = g2.x;
-                pa[c + 1] = g2.y;
-                if (ki) {
+                for (int c = 0; c < NH; c += 2) {
                     const double2 k2 = *reinterpret_cast<const double2*>(ki + c);
                     pb[c] = k2.x;
                     pb[c + 1] = k2.y;
                 }
-            }
-        } else {
+            } else {
 #pragma unroll
-            for (int c = 0; c < NH; ++c)
-                if (o0 + c < n) {
-                    pa[c] = gi[c];
-                    if (ki) pb[c] = ki[c];
-                }
+                for (int c = 0; c < NH; ++c)
+                    if (o0 + c < n) pb[c] = ki[c];
+            }
         }
         if (MODE == M_KLAST && Sg.aux)
 #pragma unroll
@@ -458,7 +453,9 @@ emu_pass_kernel(const __grid_constant__ Params ep) {
     // them back itself, so its own wait is all the synchronisation they need, and they have a
     // whole window (or the previous job's last one) to arrive.
     const int pair = lane & 7, r0 = warp * RPW + (lane >> 3);
-    unsigned char* const raw = sm + S * APL + b_bytes(KIND) + tid * 16;
+    constexpr bool ROWS = KIND == K_KIN;   // staged as whole rows, each read by the thread of its outputs
+    unsigned char* const raw = sm + S * APL + b_bytes(KIND) + (ROWS ? r0 * RAWROW + pair * 16 : tid * 16);
+    constexpr int RAWSTEP = ROWS ? 4 * RAWROW : THREADS * 16;
     EJob Q = J;
     const double* qsrc = nullptr;
     int qx = 0, qleft = 0, qn = 0;
@@ -481,7 +478,7 @@ emu_pass_kernel(const __grid_constant__ Params ep) {
             while (x >= qn) x -= qn;
 #pragma unroll
             for (int g4 = 0; g4 < RPW / 4; ++g4)
-                if (r0 + 4 * g4 < Q.lt) cp_async16(raw + g4 * THREADS * 16, qsrc + (long long)(4 * g4) * qn + x);
+                if (r0 + 4 * g4 < Q.lt) cp_async16(raw + g4 * RAWSTEP, qsrc + (long long)(4 * g4) * qn + x);
             qx += 16;
             while (qx >= qn) qx -= qn;
             --qleft;
@@ -568,7 +565,7 @@ emu_pass_kernel(const __grid_constant__ Params ep) {
                         w.v[g4][1] = __double_as_longlong(load_in<MODE>(Sg, J.orb, J.a0 + r0 + 4 * g4, x + 1));
                     } else {
                         // x is even and n is even: x + 1 is in the line, 16-byte aligned
-                        const longlong2 d2 = *reinterpret_cast<const longlong2*>(raw + g4 * THREADS * 16);
+                        const longlong2 d2 = *reinterpret_cast<const longlong2*>(raw + g4 * RAWSTEP);
                         w.v[g4][0] = d2.x;
                         w.v[g4][1] = d2.y;
                         if constexpr (INI) {
@@ -602,13 +599,53 @@ emu_pass_kernel(const __grid_constant__ Params ep) {
             };
             if constexpr (OUTI)
                 if (tid < J.lt) Sg.gout[(long long)J.orb * Sg.N + J.a0 + tid] = rowE[tid] + Ef - OUT_EXP;
+            // kinetic passes: the thread of line er, outputs 8 half .. + 7 of a window, slices the
+            // same positions of the line's slabs, and keeps them for the epilogue: the
+            // outputs of window w are the positions of slab w + 1 (pa; pn is slab w + 2)
+            double pa[NH], pn[NH];
+            auto row_slab = [&]() {
+                cp_wait<0>();
+                __syncthreads();
+                const double2* const src = reinterpret_cast<const double2*>(
+                    sm + S * APL + b_bytes(KIND) + er * RAWROW + half * 64);
+                const int E = rowE[er];
+                unsigned char* const d = Asm + (2 * slot + half) * LBOA + er * 16;
+                uint32_t h[4][S];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const double2 v = er < J.lt ? src[c] : make_double2(0.0, 0.0);
+                    pa[2 * c] = pn[2 * c];
+                    pa[2 * c + 1] = pn[2 * c + 1];
+                    pn[2 * c] = v.x;
+                    pn[2 * c + 1] = v.y;
+                    digit_pairs(quantize(v.x, E) + DBIAS, quantize(v.y, E) + DBIAS, h[c]);
+                }
+#pragma unroll
+                for (int q = 0; q < S; ++q)
+                    *reinterpret_cast<uint4*>(d + q * APL) = make_uint4(h[0][q], h[1][q], h[2][q], h[3][q]);
+                if (++slot == NSLOT) slot = 0;
+            };
             double eacc = 0.0;
             unsigned top = 0;   // largest high word of this thread's integer outputs' magnitudes
             int first = 0;   // slot of the window's first slab
 #pragma unroll 1
             for (int w = 0; w < nwin && !failed; ++w) {
                 const int o = w * N;
-                if (w == 0) {
+                if constexpr (ROWS) {
+                    if (w == 0) {
+#pragma unroll 1
+                        for (int k = 0; k < NSLOT; ++k) {
+                            row_slab();
+                            if (k + 1 < NSLOT) {
+                                __syncthreads();   // the rows are read
+                                copy_slab();
+                            }
+                        }
+                    } else {
+                        row_slab();
+                        if (++first == NSLOT) first = 0;
+                    }
+                } else if (w == 0) {
 #pragma unroll 1
                     for (int k = 0; k < NSLOT; ++k) {
                         Raw v;
@@ -622,7 +659,8 @@ emu_pass_kernel(const __grid_constant__ Params ep) {
                     if (++first == NSLOT) first = 0;
                 }
                 issue_mmas(first);
-                double pa[NH], pb[NH], pc[NH];
+                if constexpr (ROWS) copy_slab();   // (every row was read before the barrier above)
+                double pb[NH], pc[NH];
                 prefetch_epilogue<KIND, MODE>(Sg, o + NH * half, er, J.lt, J.a0, J.orb, J.grp, pa,
                                               pb, pc);
 
