@@ -113,13 +113,6 @@ struct Tune {
     bool persist = false;   // persistent double-buffered grid vs one CTA per job
 };
 
-// FP32 potential pass: compensated density sums in shared memory, one float
-// pair per (output, line) of a tile
-template <typename T>
-static size_t pot_smem(int mode, int LT, int n) {
-    return (mode == M_POT && sizeof(T) == 4) ? (size_t)LT * n * 8 : 0;
-}
-
 // one staging buffer per CTA unless it prefetches (persistent grid, or the
 // orbital walk of the potential pass)
 static int nbuf(int mode, const Tune& t) { return (t.persist || mode == M_POT) ? 2 : 1; }
@@ -176,19 +169,38 @@ static int rowlen_of(int n, int R, const KindGeom& g, size_t elt) {
     return rl;
 }
 
+// FP32 calls that pass32.cu takes: the potential pass, and the compressed passes where
+// every segment stores its whole grid.  The coefficients of a region or a box are looked up
+// one by one, which the row-wise kernel does better: 44 of 1037 us of H psi of 64 orbitals
+// on a ball in a coarse 48^3 cell.
+template <typename T>
+static bool use_pass32(const PassCall<T>& c) {
+    if (sizeof(T) != 4) return false;
+    if (c.mode == M_POT) return true;
+    if (c.mode != M_UNCOMP && c.mode != M_COMP) return false;
+    for (const auto& d : c.segs)
+        if (d.s.mapc != nullptr || d.s.bx1 != 0 || d.gn != 0) return false;
+    return true;
+}
+
 template <typename T>
 static bool tune_valid(const PassCall<T>& c, const Tune& t) {
     const KindGeom g = kind_geom(c.kind);
+    const bool p32 = use_pass32(c);
+    if (p32 && (t.R != 8 || t.LT < 8 || t.persist)) return false;
     for (const auto& d : c.segs) {
         int n, N;
         pass_dims(d.Nf, c.pass, n, N);
-        // the staging buffers (and the FP32 potential pass's density sums) must fit
-        if (nbuf(c.mode, t) * ((size_t)t.LT * rowlen_of(n, t.R, g, sizeof(T)) + 2) * sizeof(T) +
-                pot_smem<T>(c.mode, t.LT, n) > 200 * 1024)
+        if (p32) {
+            if (pass32_smem(c.kind, c.mode, t.LT, n, d.user_rho != nullptr) > 200 * 1024) return false;
+            continue;
+        }
+        // the staging buffers must fit
+        if (nbuf(c.mode, t) * ((size_t)t.LT * rowlen_of(n, t.R, g, sizeof(T)) + 2) * sizeof(T) > 200 * 1024)
             return false;
         if (c.mode == M_POT && sizeof(T) == 8) {
             const int nslots = (NTHREADS / 32) * (32 / t.LT);
-            const int cpt = pot_out<T>() / t.R;
+            const int cpt = POT_OUT / t.R;
             if ((long long)cpt * nslots < (n + t.R - 1) / t.R) return false;
         }
     }
@@ -264,6 +276,7 @@ static wvl_status exec_call(PassCall<T>& c, const Tune& tn, cudaStream_t st) {
     if (kind_geom(K_MF).hl != 8 || kind_geom(K_MFT).hl != 7)
         return fail(WVL_EUNSUPPORTED, "magic filter offset k0 = %d, kernels assume -7", filters().k0);
     const bool emu = c.emu;
+    const bool p32 = use_pass32(c);
     size_t i = 0;
     while (i < c.segs.size()) {
         PassParams<T> p;
@@ -293,7 +306,12 @@ static wvl_status exec_call(PassCall<T>& c, const Tune& tn, cudaStream_t st) {
             } else {
                 s.nwin = 1;
                 s.tiles = (s.N + tn.LT - 1) / tn.LT;
-                s.rowlen = rowlen_of(s.n, tn.R, g, sizeof(T));
+                if (!p32) s.rowlen = rowlen_of(s.n, tn.R, g, sizeof(T));
+                // the compressed form of a full grid: tiles of LT / 2 lines of two rows
+                if (p32 && c.mode != M_POT) {
+                    const int row = c.mode == M_UNCOMP ? s.N2 : s.N1, h = tn.LT / 2;
+                    s.tiles = s.N / row / 2 * ((row + h - 1) / h);
+                }
             }
             long long units = s.norb;
             if (c.mode == M_POT) {
@@ -328,7 +346,8 @@ static wvl_status exec_call(PassCall<T>& c, const Tune& tn, cudaStream_t st) {
             }
             s.blk0 = blk;
             blk += units * s.tiles;
-            if (!emu) smem = std::max(smem, (size_t)tn.LT * s.rowlen);
+            if (p32) smem = std::max(smem, pass32_smem(c.kind, c.mode, tn.LT, s.n, s.rho != nullptr));
+            else if (!emu) smem = std::max(smem, (size_t)tn.LT * s.rowlen);
             nmax = std::max(nmax, s.n);
             p.seg[k] = s;
         }
@@ -357,10 +376,16 @@ static wvl_status exec_call(PassCall<T>& c, const Tune& tn, cudaStream_t st) {
             if (e != cudaSuccess) return cuda_fail(e, "emulated pass launch");
             continue;
         }
+        if constexpr (sizeof(T) == 4)
+            if (p32) {
+                cudaError_t e = launch_pass32(c.kind, c.mode, p, blk, pass32_threads(tn.LT, nmax), smem, st);
+                if (e != cudaSuccess) return cuda_fail(e, "pass launch");
+                continue;
+            }
         // two staging buffers, each rounded to 16 bytes
         const size_t per16 = 16 / sizeof(T);
         p.bufelems = (int)((smem + per16 - 1) / per16 * per16);
-        smem = nbuf(c.mode, tn) * (size_t)p.bufelems * sizeof(T) + pot_smem<T>(c.mode, tn.LT, nmax);
+        smem = nbuf(c.mode, tn) * (size_t)p.bufelems * sizeof(T);
         cudaError_t e = launch_pass<T>(c.kind, c.mode, tn.R, p, blk, smem, st, tn.persist);
         if (e != cudaSuccess) return cuda_fail(e, "pass launch");
     }
@@ -2091,7 +2116,9 @@ static wvl_status plan_exec(wvl_plan* plan, const void* psi, const void* const* 
     const unsigned long long before = g_launches.load();
     // capture the enqueue sequence into a graph; the kernels' shared-memory
     // attributes are set before capture (host-only calls)
-    cudaError_t e = (plan->prec == WVL_F64_EMU) ? prepare_emu_kernels() : prepare_pass_kernels<T>();
+    cudaError_t e;
+    e = (plan->prec == WVL_F64_EMU) ? prepare_emu_kernels() : prepare_pass_kernels<T>();
+    if (sizeof(T) == 4 && e == cudaSuccess) e = prepare_pass32();
     if (e == cudaSuccess && plan->prec != WVL_F64_EMU) e = prepare_fused_kernels<T>();
     if (e != cudaSuccess) return cuda_fail(e, "kernel attributes");
     cudaGraph_t g = nullptr;

@@ -39,9 +39,8 @@ enum Mode {
 constexpr int MAXSEG = 8;      // cells (segments) per launch
 constexpr int NTHREADS = 128;  // threads per CTA (4 warps)
 // register-resident density outputs per thread in the FP64 M_POT pass (the
-// FP32 pass keeps its compensated density sums in shared memory)
-template <typename T>
-__host__ __device__ constexpr int pot_out() { return sizeof(T) == 8 ? 32 : 16; }
+// FP32 pass, pass32.cu, keeps its compensated density sums in shared memory)
+constexpr int POT_OUT = 32;
 constexpr int MAX_FINE = 1024; // largest fine extent of one axis
 
 // One cell's orbitals inside one pass launch.  Element offsets are per
@@ -234,6 +233,14 @@ void fill_taps(PassParams<T>& p, int kind, double hgrid);
 template <typename T>
 cudaError_t launch_pass(int kind, int mode, int R, const PassParams<T>& p,
                         long long nunits, size_t smem, cudaStream_t st, bool persistent);
+
+// The FP32 passes of pass32.cu: threads and shared memory of a launch whose longest
+// output line is n (rho: the potential pass has density sums), and the launch.
+int pass32_threads(int LT, int nmax);
+size_t pass32_smem(int kind, int mode, int LT, int n, bool rho);
+cudaError_t launch_pass32(int kind, int mode, const PassParams<float>& p, long long nunits, int threads,
+                          size_t smem, cudaStream_t st);
+cudaError_t prepare_pass32();
 
 // Sets the dynamic shared-memory attribute of every pass kernel on the
 // current device (done lazily by launch_pass too; needed before capture).
