@@ -1002,7 +1002,7 @@ static wvl_status run_fused(int op, std::vector<CellRun<T>>& runs, Prof* prof, c
                     break;
                 const bool plane = prog == FZ_SKM12 || prog == FZ_MFTA12;
                 // one launch shape per launch of a plane kernel
-                const FzShape shape = fz_plane_shape<T>(r.Nf[0], r.Nf[1], (long long)r.norb * r.Nf[2]);
+                const FzShape shape = fz_plane_shape<T>(prog, r.Nf[0], r.Nf[1], (long long)r.norb * r.Nf[2]);
                 if (k > 0 && plane && shape != p.shape) break;
                 p.shape = shape;
                 FzSeg<T>& s = p.seg[k];

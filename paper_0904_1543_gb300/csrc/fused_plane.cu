@@ -1,0 +1,502 @@
+// The plane kernels of the fused chain (fused_kernel.cu) for square FP32 planes of 32, 64, 96 or
+// 128 points a side: most filters are applied along the buffer's rows of 16-byte words ("line
+// items": 16 consecutive outputs of two neighbouring lines per thread), the plane being
+// transposed between the filters of different axes as the outputs are stored.
+//
+// A plane kernel is a chain of phases between barriers, each bound half by the FMA pipe and
+// half by its latencies (load, window, stores), so what counts is how much of a phase
+// another one covers.  The swizzled buffers need no padding, so three 96^2 planes share an SM
+// (two in the general form); 128^2 planes are alone on their SM, and a CTA per SM walks
+// over them with a third buffer for the next plane.  Two values of a row are the operands
+// of a packed FMA as they are loaded; a row item has to copy each value into both
+// halves.  Extents are compile-time constants, which leaves one XOR per 16-byte load of address
+// arithmetic.  Microseconds of SYN3 + SKM12 / MFTA12 in the general form and here: 128^2 (48
+// orbitals) 812 / 432 and 688 / 330 (746 / 388 with extents from memory), 96^2 (64) 456 /
+// 219 and 388 / -, 64^2 (128) 267 / 123 and 246 / -, 32^2 (512) 150 / 78 and 129 / -.  MFTA12 on
+// smaller planes stays with the general form, whose CTAs need two buffers where this one
+// needs three.  Also tried at 128^2, with extents from memory: items of four lines (256
+// threads: 760 / 447), T_2 as items along the contiguous axis of a transposed s (800 to 820),
+// a warp of its own for the copies (1153 / 1205: one warp's copies in flight are too few).
+//
+// The outputs' sums keep the order of the general form except MFT_1 and MFT_2, whose order
+// is exchanged; t and Ekin are the same bits.
+#include <algorithm>
+#include <type_traits>
+
+#include "fused.cuh"
+
+namespace wvl {
+namespace {
+
+// A buffer holds a plane as [row][col], RS floats per row, one buffer after
+// the other.  The 16-byte word u of row j lies at word u ^ swz(j), so that
+// eight lanes find distinct banks on consecutive words of a row, on one word of eight
+// consecutive rows and on one word of eight rows four apart.
+//   8 i + j -> j ^ (i & 3):  bijective in the low three bits of the row and in bits 2 to 4
+__device__ __forceinline__ unsigned swz(int row) { return (unsigned)((row & 7) ^ ((row >> 3) & 3)); }
+
+__host__ __device__ constexpr int floor8(int d) { return d >= 0 ? d / 8 : -((7 - d) / 8); }
+
+template <int RS>
+struct PlaneBuf {
+    static constexpr unsigned ROW = RS * 4, SIZE = RS * ROW;   // bytes
+};
+
+extern __shared__ __align__(1024) unsigned char fsm[];
+
+__device__ __forceinline__ float4& word(unsigned off) { return *reinterpret_cast<float4*>(fsm + off); }
+__device__ __forceinline__ float2& half_word(unsigned off) { return *reinterpret_cast<float2*>(fsm + off); }
+
+// LP neighbouring values (2 or 4) of a row, as pairs
+template <int LP>
+__device__ __forceinline__ void load_lines(unsigned off, float2 (&v)[LP / 2]) {
+    if constexpr (LP == 4) {
+        const float4 q = word(off);
+        v[0] = make_float2(q.x, q.y);
+        v[1] = make_float2(q.z, q.w);
+    } else {
+        v[0] = half_word(off);
+    }
+}
+// byte offset of lines LP u .. in a row of the block of eight rows q, row 0 of the block
+template <int LP>
+__device__ __forceinline__ unsigned line_off(int u, int q) {
+    if constexpr (LP == 4) return (unsigned)(u ^ (q & 3)) << 4;
+    else return ((unsigned)((u >> 1) ^ (q & 3)) << 4) + ((u & 1) << 3);
+}
+// NO outputs from NO kb on (along the rows of the buffer at buf, periodic with 8 nb) of the
+// lines LP u ..:  acc[k] = sum_t f[k & 1][t] row(NO kb + k - HL + off(k & 1) + t)
+// td: the taps, each twice
+template <int KIND, int RS, int LP, int NO = 16>
+__device__ __forceinline__ void line_item(unsigned buf, int kb, int nb, int u, const float2 (&td)[2][32],
+                                          float2 (&acc)[NO][LP / 2]) {
+    constexpr int NT = KT<KIND>::NT, HL = KT<KIND>::HL, W = NO + NT - 1 + KT<KIND>::EXTRA;
+    constexpr unsigned ROW = PlaneBuf<RS>::ROW;
+    constexpr int B0 = floor8(-HL), NB = floor8(W - 1 - HL) - B0 + 1;
+    unsigned T[NB];   // the lines' values in the first row of the window's blocks of eight
+    #pragma unroll
+    for (int b = 0; b < NB; ++b) {
+        int q = NO / 8 * kb + B0 + b;
+        q += q < 0 ? nb : 0;
+        q -= q >= nb ? nb : 0;
+        T[b] = buf + q * 8 * ROW + line_off<LP>(u, q);
+    }
+    #pragma unroll
+    for (int k = 0; k < NO; ++k)
+        #pragma unroll
+        for (int m = 0; m < LP / 2; ++m) acc[k][m] = make_float2(0.f, 0.f);
+    static_for<W>([&](auto jc) {
+        constexpr int j = decltype(jc)::value, d = j - HL, i = d - 8 * floor8(d);
+        float2 v[LP / 2];
+        load_lines<LP>((T[floor8(d) - B0] ^ (i << 4)) + i * ROW, v);
+        static_for<NO>([&](auto kc) {
+            constexpr int k = decltype(kc)::value;
+            constexpr int t = j - k - ((k & 1) ? KT<KIND>::OFF1 : KT<KIND>::OFF0);
+            // (the other filters' parities are equal)
+            constexpr int e = KIND == K_SYN || KIND == K_ANA ? k & 1 : 0;
+            if constexpr (tap_on<KIND>(t)) {
+                #pragma unroll
+                for (int m = 0; m < LP / 2; ++m) acc[k][m] = __ffma2_rn(td[e][t], v[m], acc[k][m]);
+            }
+        });
+    });
+}
+// the item's outputs, transposed: line LP u + e becomes a row, its words 4 kb + h
+template <int RS, int LP>
+__device__ __forceinline__ unsigned trans_base(unsigned buf, int kb, int u) {
+    const int s = LP == 4 ? (4 * (u & 1)) ^ ((u >> 1) & 3) : (2 * (u & 3)) ^ ((u >> 2) & 3);
+    return buf + LP * u * PlaneBuf<RS>::ROW + ((unsigned)((4 * kb) ^ s) << 4);
+}
+template <int RS>
+__device__ __forceinline__ float4& trans_word(unsigned base, int e, int h) {
+    return word((base ^ ((e ^ h) << 4)) + e * PlaneBuf<RS>::ROW);
+}
+// outputs 4 h .. 4 h + 3 of line e
+template <int LP>
+__device__ __forceinline__ float4 line_word(const float2 (&acc)[16][LP / 2], int e, int h) {
+    float q[4];
+    #pragma unroll
+    for (int k = 0; k < 4; ++k) q[k] = (e & 1) ? acc[4 * h + k][e / 2].y : acc[4 * h + k][e / 2].x;
+    return make_float4(q[0], q[1], q[2], q[3]);
+}
+template <int RS, int LP>
+__device__ __forceinline__ void store_trans(unsigned buf, int kb, int u, const float2 (&acc)[16][LP / 2]) {
+    const unsigned base = trans_base<RS, LP>(buf, kb, u);
+    #pragma unroll
+    for (int e = 0; e < LP; ++e)
+        #pragma unroll
+        for (int h = 0; h < 4; ++h) trans_word<RS>(base, e, h) = line_word<LP>(acc, e, h);
+}
+// the item's outputs to the global plane of N columns at g
+template <int LP>
+__device__ __forceinline__ void store_global(float* g, int N, int kb, int u, const float2 (&acc)[16][LP / 2]) {
+    g += (long long)(16 * kb) * N + LP * u;
+    #pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        if constexpr (LP == 4)
+            *reinterpret_cast<float4*>(g + (long long)k * N) =
+                make_float4(acc[k][0].x, acc[k][0].y, acc[k][LP / 2 - 1].x, acc[k][LP / 2 - 1].y);
+        else
+            *reinterpret_cast<float2*>(g + (long long)k * N) = acc[k][0];
+    }
+}
+// word i (0 to 3) of chunk a (16 columns) of row: (chunk_base(row, a) ^ (i << 4))
+template <int RS>
+__device__ __forceinline__ unsigned chunk_base(unsigned buf, int row, int a) {
+    const unsigned s = swz(row);
+    return buf + row * PlaneBuf<RS>::ROW + ((unsigned)(a ^ (int)(s >> 2)) << 6) + ((s & 3) << 4);
+}
+
+// Row `row` (periodic with 16 nch columns) from HLR columns before chunk ch on: the window of
+// the chunk's outputs
+template <int KIND>
+struct RowWin {
+    static constexpr int HLR = (KT<KIND>::HL + 3) / 4 * 4, D = HLR - KT<KIND>::HL;
+    static constexpr int WV = (16 + KT<KIND>::NT - 1 + KT<KIND>::EXTRA + D + 3) / 4;
+};
+template <int KIND, int RS>
+__device__ __forceinline__ void row_win(unsigned buf, int row, int ch, int nch, float (&win)[4 * RowWin<KIND>::WV]) {
+    constexpr int HU = RowWin<KIND>::HLR / 4, G = (HU + 3) / 4, PH = 4 * G - HU;
+    constexpr int WV = RowWin<KIND>::WV, NG = (PH + WV + 3) / 4;
+    unsigned T[NG];
+    #pragma unroll
+    for (int g = 0; g < NG; ++g) {
+        int a = ch - G + g;
+        a += a < 0 ? nch : 0;
+        a -= a >= nch ? nch : 0;
+        T[g] = chunk_base<RS>(buf, row, a);
+    }
+    static_for<WV>([&](auto qc) {
+        constexpr int q = decltype(qc)::value + PH, w = 4 * decltype(qc)::value;
+        const float4 v = word(T[q / 4] ^ ((q % 4) << 4));
+        win[w] = v.x;
+        win[w + 1] = v.y;
+        win[w + 2] = v.z;
+        win[w + 3] = v.w;
+    });
+}
+// the chunk's outputs; D: the filter's first window element
+template <int KIND, int D, int NW>
+__device__ __forceinline__ void row_fir(const float (&win)[NW], const float2 (&tp)[32], float (&acc)[16]) {
+    #pragma unroll
+    for (int k = 0; k < 16; ++k) acc[k] = 0.f;
+    const float none[2][32] = {};   // (scalar taps: not used in FP32)
+    fir<float, KIND, 16, D>(win, none, tp, acc);
+}
+template <int RS>
+__device__ __forceinline__ void store_chunk(unsigned buf, int row, int ch, const float (&v)[16]) {
+    const unsigned b = chunk_base<RS>(buf, row, ch);
+    #pragma unroll
+    for (int q = 0; q < 4; ++q) word(b ^ (q << 4)) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+}
+
+// a job: one fine-grid plane (RS x RS) of an orbital
+struct Plane {
+    const FzSeg<float>* S;
+    int I3, o;
+    long long base;   // of the plane in the fine arrays
+};
+__device__ __forceinline__ Plane plane_of(const FzTileParams& p, long long job) {
+    int si = 0;
+    #pragma unroll 1
+    while (si + 1 < p.nseg && job >= p.seg[si + 1].blk0) ++si;
+    Plane q;
+    q.S = &p.seg[si];
+    const long long loc = job - q.S->blk0;
+    q.I3 = (int)(loc % q.S->N3);
+    q.o = (int)(loc / q.S->N3);
+    q.base = (long long)q.o * q.S->P + (long long)q.I3 * q.S->N1 * q.S->N2;
+    return q;
+}
+// starts the copy of the plane at src -> buf as [I2][I1]
+template <int RS>
+__device__ __forceinline__ void fetch_plane(unsigned buf, const float* src) {
+    const int lane = threadIdx.x & 31, nw = (int)(blockDim.x >> 5);
+    #pragma unroll 1
+    for (int r = threadIdx.x >> 5; r < RS; r += nw) {
+        const unsigned s = swz(r);
+        for (int u = lane; u < RS / 4; u += 32)
+            cp_async16(&word(buf + r * PlaneBuf<RS>::ROW + ((u ^ s) << 4)), src + r * RS + 4 * u);
+    }
+}
+
+// Items i, i + step, ... of an na x nb grid (b fastest), without a division per item
+struct Walk {
+    int a, b, da, db, na, nb;
+    __device__ __forceinline__ Walk(int i, int step, int na_, int nb_)
+        : a(i / nb_), b(i - a * nb_), da(step / nb_), db(step - da * nb_), na(na_), nb(nb_) {}
+    template <typename F>
+    __device__ __forceinline__ void each(F&& f) const {
+        int x = a, y = b;
+        #pragma unroll 1
+        while (x < na) {
+            f(x, y);
+            x += da;
+            y += db;
+            if (y >= nb) {
+                y -= nb;
+                ++x;
+            }
+        }
+    }
+};
+
+// one CTA per SM fetches the next plane while it filters this one; smaller planes have other
+// CTAs on their SM for that
+__host__ __device__ constexpr bool prefetches(int rs) { return rs == 128; }
+
+template <int PROG, int RS, int REGS, int LP>
+__global__ void __maxnreg__(REGS) fz_tplane_kernel(const __grid_constant__ FzTileParams p) {
+    __shared__ double red[FZ_PTHREADS / 32];
+    unsigned X = 0, Z = 2 * PlaneBuf<RS>::SIZE;
+    constexpr unsigned Y = PlaneBuf<RS>::SIZE;
+    constexpr int N1 = RS, N2 = RS;
+    const int T = (int)blockDim.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = T >> 5;
+
+    Plane c = plane_of(p, blockIdx.x);
+    fetch_plane<RS>(X, c.S->in + c.base);
+    cp_commit();
+    if (PROG == FZ_MFTA12) {
+        fetch_plane<RS>(Z, c.S->in2 + c.base);
+        cp_commit();
+    }
+    #pragma unroll 1
+    for (long long job = blockIdx.x; job < p.njobs; job += gridDim.x) {
+        const FzSeg<float>& S = *c.S;
+        // items along axis 2 ([I2][I1] planes) and along axis 1 ([I1][I2])
+        const int nb2 = N2 / 8, nb1 = N1 / 8;
+        const Walk w2(threadIdx.x, T, N2 / 16, N1 / LP), w1(threadIdx.x, T, N1 / 16, N2 / LP);
+        const bool more = job + gridDim.x < p.njobs;
+        Plane nx = c;
+        if (more) nx = plane_of(p, job + gridDim.x);
+        float2 acc[16][LP / 2];
+
+        if constexpr (PROG == FZ_SKM12) {
+            cp_wait<0>();
+            __syncthreads();   // the plane is here, and the last one is done with
+            if (more) {
+                fetch_plane<RS>(Z, nx.S->in + nx.base);
+                cp_commit();
+            }
+            // s = S_1 S_2 a -> X
+            w2.each([&](int kb, int u) {
+                line_item<K_SYN, RS, LP>(X, kb, nb2, u, p.td[0], acc);
+                store_trans<RS, LP>(Y, kb, u, acc);
+            });
+            __syncthreads();
+            w1.each([&](int kb, int u) {
+                line_item<K_SYN, RS, LP>(Y, kb, nb1, u, p.td[0], acc);
+                store_trans<RS, LP>(X, kb, u, acc);
+            });
+            __syncthreads();
+            // eight rows of four columns, as in the general form: the same chains of Ekin
+            const Walk we(threadIdx.x, T, N2 / 8, N1 / 4);
+            EAcc<float> e;
+            // t = MF_2 (MF_1 s in Y), out
+            auto put_t = [&](int kb, int u) {
+                float2 m[8][2];
+                line_item<K_MF, RS, 4, 8>(Y, kb, nb2, u, p.td[3], m);
+                float* const g = S.out3 + c.base + (long long)(8 * kb) * N1 + 4 * u;
+                #pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    *reinterpret_cast<float4*>(g + (long long)k * N1) = make_float4(m[k][0].x, m[k][0].y, m[k][1].x, m[k][1].y);
+            };
+            // v = T_2 s + T_1 s, out if asked for, and its part <s, v>; t1(k): T_1 s at row k
+            auto put_v = [&](int kb, int u, auto&& t1) {
+                float2 m[8][2];
+                line_item<K_KIN, RS, 4, 8>(X, kb, nb2, u, p.td[2], m);
+                const unsigned o = X + kb * 8 * PlaneBuf<RS>::ROW + line_off<4>(u, kb);
+                float ei = 0.f;
+                #pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const float4 s = word((o ^ (k << 4)) + k * PlaneBuf<RS>::ROW), a = t1(k);
+                    const float4 v = make_float4(m[k][0].x + a.x, m[k][0].y + a.y, m[k][1].x + a.z, m[k][1].y + a.w);
+                    ei = fmaf(s.x, v.x, ei);
+                    ei = fmaf(s.y, v.y, ei);
+                    ei = fmaf(s.z, v.z, ei);
+                    ei = fmaf(s.w, v.w, ei);
+                    if (S.out2 != nullptr)
+                        *reinterpret_cast<float4*>(S.out2 + c.base + (long long)(8 * kb + k) * N1 + 4 * u) = v;
+                }
+                e.add(ei);
+            };
+            const int nch = N1 / 16;
+            const Walk wr(warp, nw, nch, N2 / 32);   // chunks of 16 columns, blocks of 32 rows
+            if (S.part != nullptr && S.out2 != nullptr) {
+                // H psi: T_1 s -> v and MF_1 s -> Y from one window
+                wr.each([&](int ch, int rb) {
+                    const int row = rb * 32 + lane;
+                    float win[4 * RowWin<K_KIN>::WV], v[16];
+                    row_win<K_KIN, RS>(X, row, ch, nch, win);
+                    row_fir<K_KIN, RowWin<K_KIN>::D>(win, p.tp[0], v);
+                    if constexpr (prefetches(RS)) {
+                        // through the item's own place in Y, so that four lanes write 64 bytes
+                        // of a row: 128^2 746 against 797, 96^2 425 against 414
+                        store_chunk<RS>(Y, row, ch, v);
+                        __syncwarp();
+                        #pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const int r = rb * 32 + 8 * i + ((lane >> 2 & 1) << 2) + (lane >> 3), q = lane & 3;
+                            *reinterpret_cast<float4*>(S.out2 + c.base + (long long)r * N1 + 16 * ch + 4 * q) =
+                                word(chunk_base<RS>(Y, r, ch) ^ (q << 4));
+                        }
+                        __syncwarp();
+                    } else {
+                        float4* const g = reinterpret_cast<float4*>(S.out2 + c.base + (long long)row * N1 + 16 * ch);
+                        #pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            g[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                    }
+                    row_fir<K_MF, RowWin<K_KIN>::HLR - KT<K_MF>::HL>(win, p.tp[1], v);
+                    store_chunk<RS>(Y, row, ch, v);
+                });
+                __syncthreads();
+                we.each([&](int kb, int u) {
+                    put_t(kb, u);
+                    const float* const g = S.out2 + c.base + (long long)(8 * kb) * N1 + 4 * u;
+                    float4 t1[8];
+                    #pragma unroll
+                    for (int k = 0; k < 8; ++k) t1[k] = *reinterpret_cast<const float4*>(g + (long long)k * N1);
+                    put_v(kb, u, [&](int k) { return t1[k]; });
+                });
+            } else {
+                if (S.part != nullptr) {
+                    wr.each([&](int ch, int rb) {
+                        const int row = rb * 32 + lane;
+                        float win[4 * RowWin<K_KIN>::WV], v[16];
+                        row_win<K_KIN, RS>(X, row, ch, nch, win);
+                        row_fir<K_KIN, RowWin<K_KIN>::D>(win, p.tp[0], v);
+                        store_chunk<RS>(Y, row, ch, v);
+                    });
+                    __syncthreads();
+                    we.each([&](int kb, int u) {
+                        const unsigned o = Y + kb * 8 * PlaneBuf<RS>::ROW + line_off<4>(u, kb);
+                        put_v(kb, u, [&](int k) { return word((o ^ (k << 4)) + k * PlaneBuf<RS>::ROW); });
+                    });
+                    __syncthreads();
+                }
+                wr.each([&](int ch, int rb) {
+                    const int row = rb * 32 + lane;
+                    float win[4 * RowWin<K_MF>::WV], v[16];
+                    row_win<K_MF, RS>(X, row, ch, nch, win);
+                    row_fir<K_MF, RowWin<K_MF>::D>(win, p.tp[1], v);
+                    store_chunk<RS>(Y, row, ch, v);
+                });
+                __syncthreads();
+                we.each([&](int kb, int u) { put_t(kb, u); });
+            }
+            if (S.part != nullptr) {
+                const double tot = fz_block_sum(e, red);
+                if (threadIdx.x == 0) S.part[(long long)c.o * S.ptiles + S.poff + c.I3] = tot;
+            }
+        } else {
+            cp_wait<1>();      // x; v may still be under way
+            __syncthreads();
+            // w = MFT_1 MFT_2 x + v -> X as [I2][I1]
+            w2.each([&](int kb, int u) {
+                line_item<K_MFT, RS, LP>(X, kb, nb2, u, p.td[0], acc);
+                store_trans<RS, LP>(Y, kb, u, acc);
+            });
+            cp_wait<0>();
+            __syncthreads();
+            w1.each([&](int kb, int u) {
+                line_item<K_MFT, RS, LP>(Y, kb, nb1, u, p.td[0], acc);
+                const unsigned bx = trans_base<RS, LP>(X, kb, u), bz = trans_base<RS, LP>(Z, kb, u);
+                #pragma unroll
+                for (int e = 0; e < LP; ++e)
+                    #pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        const float4 v = trans_word<RS>(bz, e, h), m = line_word<LP>(acc, e, h);
+                        trans_word<RS>(bx, e, h) = make_float4(m.x + v.x, m.y + v.y, m.z + v.z, m.w + v.w);
+                    }
+            });
+            __syncthreads();
+            if (more) fetch_plane<RS>(Z, nx.S->in + nx.base);
+            cp_commit();
+            // w' = A_2 A_1 w, A_1 with a lane per I2, chunks of 16
+            const int nch = N1 / 16;
+            const Walk wr(warp, nw, nch, N2 / 32);
+            wr.each([&](int ch, int rb) {
+                const int row = rb * 32 + lane;
+                float win[4 * RowWin<K_ANA>::WV], v[16];
+                row_win<K_ANA, RS>(X, row, ch, nch, win);
+                row_fir<K_ANA, RowWin<K_ANA>::D>(win, p.tp[0], v);
+                store_chunk<RS>(Y, row, ch, v);
+            });
+            __syncthreads();
+            if (more) fetch_plane<RS>(X, nx.S->in2 + nx.base);
+            cp_commit();
+            w2.each([&](int kb, int u) {
+                line_item<K_ANA, RS, LP>(Y, kb, nb2, u, p.td[1], acc);
+                store_global<LP>(S.out + c.base, N1, kb, u, acc);
+            });
+        }
+        c = nx;
+        const unsigned t = X;
+        X = Z;
+        Z = t;
+    }
+}
+
+template <typename F>
+cudaError_t tplane_pick(int prog, FzShape s, F&& f) {
+    if (prog == FZ_MFTA12 && s.rs == 128) return f(fz_tplane_kernel<FZ_MFTA12, 128, 128, 2>);
+    if (prog != FZ_SKM12) return cudaErrorInvalidConfiguration;
+    switch (s.rs) {
+    case 128: return f(fz_tplane_kernel<FZ_SKM12, 128, 128, 2>);
+    case 96: return f(fz_tplane_kernel<FZ_SKM12, 96, 128, 2>);
+    case 64: return f(fz_tplane_kernel<FZ_SKM12, 64, 96, 2>);
+    case 32: return f(fz_tplane_kernel<FZ_SKM12, 32, 96, 2>);
+    }
+    return cudaErrorInvalidConfiguration;
+}
+size_t tplane_smem(FzShape s) { return (prefetches(s.rs) ? 3 : 2) * (size_t)s.rs * s.rs * sizeof(float); }
+
+}  // namespace
+
+FzShape fz_tplane_shape(int prog, int N1, int N2) {
+    const int rs = N1;
+    if (N1 != N2 || N1 % 32 != 0 || (prog == FZ_MFTA12 && rs < 128)) return {};
+    return {rs == 128 ? 512 : rs == 96 ? 160 : rs == 64 ? 128 : 32, 0, rs};
+}
+
+cudaError_t prepare_tplane(int prog, FzShape s) {
+    return tplane_pick(prog, s, [&](auto* k) {
+        return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tplane_smem(s));
+    });
+}
+
+cudaError_t launch_tplane(int prog, const FzParams<float>& p, cudaStream_t st) {
+    FzTileParams q;
+    const int nk = prog == FZ_SKM12 ? 4 : 2;
+    for (int m = 0; m < nk; ++m)
+        for (int e = 0; e < 2; ++e)
+            for (int t = 0; t < 32; ++t) q.td[m][e][t] = make_float2(p.tap[m][e][t], p.tap[m][e][t]);
+    if (prog == FZ_SKM12) {
+        tap_pairs<K_KIN>(p.tap[1], q.tp[0]);
+        tap_pairs<K_MF>(p.tap[3], q.tp[1]);
+    } else {
+        tap_pairs<K_ANA>(p.tap[1], q.tp[0]);
+    }
+    q.njobs = p.njobs;
+    q.nseg = p.nseg;
+    for (int k = 0; k < p.nseg; ++k) q.seg[k] = p.seg[k];
+    cudaError_t e = prepare_tplane(prog, p.shape);
+    if (e != cudaSuccess) return e;
+    return tplane_pick(prog, p.shape, [&](auto* k) {
+        long long grid = p.njobs;
+        if (prefetches(p.shape.rs)) {
+            int dev = 0, nsm = 0;
+            cudaError_t r = cudaGetDevice(&dev);
+            if (r == cudaSuccess) r = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+            if (r != cudaSuccess) return r;
+            grid = std::min(grid, (long long)nsm);
+        }
+        k<<<dim3((unsigned)grid), dim3(p.shape.threads), tplane_smem(p.shape), st>>>(q);
+        count_launches(1);
+        return cudaGetLastError();
+    });
+}
+
+}  // namespace wvl

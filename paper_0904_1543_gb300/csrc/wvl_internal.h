@@ -158,10 +158,13 @@ struct FzSeg {
     int RS;               // shared-memory row stride in elements
 };
 
-// Threads and register cap of a plane kernel (fz_plane_shape).
+// Launch shape of a plane kernel (fz_plane_shape): threads, register cap, and the row length of
+// the transposing form's buffers (fused_plane.cu; 0: the general form).
 struct FzShape {
-    int threads, regs;
-    bool operator!=(const FzShape& o) const { return threads != o.threads || regs != o.regs; }
+    int threads = 0, regs = 0, rs = 0;
+    bool operator!=(const FzShape& o) const {
+        return threads != o.threads || regs != o.regs || rs != o.rs;
+    }
 };
 
 template <typename T>
@@ -174,6 +177,19 @@ struct FzParams {
     FzSeg<T> seg[MAXSEG];
 };
 
+// Parameters of the transposing plane kernels: every tap twice (packed FMAs on two lines)
+struct FzTileParams {
+    float2 td[4][2][32];
+    float2 tp[2][32];     // the row filters' tap pairs of outputs 2m, 2m + 1
+    long long njobs;
+    int nseg;
+    FzSeg<float> seg[MAXSEG];
+};
+// the launch shape of a program on planes of N1 x N2 (rs = 0: not taken)
+FzShape fz_tplane_shape(int prog, int N1, int N2);
+cudaError_t launch_tplane(int prog, const FzParams<float>& p, cudaStream_t st);
+cudaError_t prepare_tplane(int prog, FzShape s);
+
 // shared-memory row stride of an xy plane with N1 columns: a 16-byte multiple
 // whose count of 16-byte words is odd (lane-per-row vector loads hit distinct banks)
 template <typename T>
@@ -183,7 +199,9 @@ inline int fz_plane_rs(int N1) {
     if ((w & 1) == 0) ++w;
     return w * v;
 }
-// Threads and register cap of a plane kernel, by the CTAs whose two planes fit in an
+// Square FP32 planes of 32 to 128 points a side in steps of 32 take the transposing form
+// (fused_plane.cu, with both sides measured).  The others: threads and register cap of a
+// plane kernel, by the CTAs whose two planes fit in an
 // SM's shared memory.  FP32, microseconds of SYN3 + SKM12 / MFTA12 per call of 64 orbitals
 // (48 at 128^2, 128 at 64^2, 256 at 48^2, 512 at 32^2):
 //   one CTA       512 threads, 128 registers: 128^2 812 / 432 (256 threads 825 / 463), 120^2
@@ -200,9 +218,11 @@ inline int fz_plane_rs(int N1) {
 // at 112 registers leave one CTA per SM: 579 / 338).  Launches of at most two CTAs per SM keep
 // 256 threads: there a plane's own time counts.  FP64 planes are bound by the FP64 pipe.
 template <typename T>
-inline FzShape fz_plane_shape(int N1, int N2, long long planes) {
+inline FzShape fz_plane_shape(int prog, int N1, int N2, long long planes) {
     if (sizeof(T) == 8) return {256, 255};
     if (planes <= 2 * 152) return {256, 128};
+    const FzShape ts = fz_tplane_shape(prog, N1, N2);
+    if (ts.rs > 0) return ts;
     const int smem = 2 * N2 * fz_plane_rs<T>(N1) * (int)sizeof(T) + 2048;
     const int ctas = 227 * 1024 / smem;
     const int items = (N2 / FZ_RC) * (N1 * (int)sizeof(T) / 16);
