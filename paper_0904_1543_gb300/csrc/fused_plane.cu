@@ -7,16 +7,16 @@
 // half by its latencies (load, window, stores), so what counts is how much of a phase
 // another one covers.  The swizzled buffers need no padding, so three 96^2 planes share an SM
 // (two in the general form); 128^2 planes are alone on their SM, and a CTA per SM walks
-// over them with a third buffer for the next plane.  Two values of a row are the operands
+// over them with a third buffer for the next plane (fz_tplane_shape).  Two values of a row are the operands
 // of a packed FMA as they are loaded; a row item has to copy each value into both
 // halves.  Extents are compile-time constants, which leaves one XOR per 16-byte load of address
 // arithmetic.  Microseconds of SYN3 + SKM12 / MFTA12 in the general form and here: 128^2 (48
 // orbitals) 812 / 432 and 688 / 330 (746 / 388 with extents from memory), 96^2 (64) 456 /
-// 219 and 388 / -, 64^2 (128) 267 / 123 and 246 / -, 32^2 (512) 150 / 78 and 129 / -.  MFTA12 on
-// smaller planes stays with the general form, whose CTAs need two buffers where this one
-// needs three.  Also tried at 128^2, with extents from memory: items of four lines (256
-// threads: 760 / 447), T_2 as items along the contiguous axis of a transposed s (800 to 820),
-// a warp of its own for the copies (1153 / 1205: one warp's copies in flight are too few).
+// 219 and 388 / 207, 64^2 (128) 267 / 123 and 239 / 119, 32^2 (512) 150 / 78 and 125 / 78 (so
+// MFTA12 keeps the general form there).  Also tried at 128^2, with extents from memory: items of
+// four lines (256 threads: 760 / 447), T_2 as items along the contiguous axis of a transposed s
+// (800 to 820), a warp of its own for the copies (1153 / 1205: one warp's copies in flight
+// are too few).
 //
 // The outputs' sums keep the order of the general form except MFT_1 and MFT_2, whose order
 // is exchanged; t and Ekin are the same bits.
@@ -241,10 +241,6 @@ struct Walk {
     }
 };
 
-// one CTA per SM fetches the next plane while it filters this one; smaller planes have other
-// CTAs on their SM for that
-__host__ __device__ constexpr bool prefetches(int rs) { return rs == 128; }
-
 template <int PROG, int RS, int REGS, int LP>
 __global__ void __maxnreg__(REGS) fz_tplane_kernel(const __grid_constant__ FzTileParams p) {
     __shared__ double red[FZ_PTHREADS / 32];
@@ -330,7 +326,7 @@ __global__ void __maxnreg__(REGS) fz_tplane_kernel(const __grid_constant__ FzTil
                     float win[4 * RowWin<K_KIN>::WV], v[16];
                     row_win<K_KIN, RS>(X, row, ch, nch, win);
                     row_fir<K_KIN, RowWin<K_KIN>::D>(win, p.tp[0], v);
-                    if constexpr (prefetches(RS)) {
+                    if constexpr (RS == 128) {
                         // through the item's own place in Y, so that four lanes write 64 bytes
                         // of a row: 128^2 746 against 797, 96^2 425 against 414
                         store_chunk<RS>(Y, row, ch, v);
@@ -441,24 +437,36 @@ __global__ void __maxnreg__(REGS) fz_tplane_kernel(const __grid_constant__ FzTil
 
 template <typename F>
 cudaError_t tplane_pick(int prog, FzShape s, F&& f) {
-    if (prog == FZ_MFTA12 && s.rs == 128) return f(fz_tplane_kernel<FZ_MFTA12, 128, 128, 2>);
-    if (prog != FZ_SKM12) return cudaErrorInvalidConfiguration;
-    switch (s.rs) {
-    case 128: return f(fz_tplane_kernel<FZ_SKM12, 128, 128, 2>);
-    case 96: return f(fz_tplane_kernel<FZ_SKM12, 96, 128, 2>);
-    case 64: return f(fz_tplane_kernel<FZ_SKM12, 64, 96, 2>);
-    case 32: return f(fz_tplane_kernel<FZ_SKM12, 32, 96, 2>);
-    }
+    if (prog == FZ_SKM12) switch (s.rs) {
+        case 128: return f(fz_tplane_kernel<FZ_SKM12, 128, 128, 2>);
+        case 96: return f(fz_tplane_kernel<FZ_SKM12, 96, 128, 2>);
+        case 64: return f(fz_tplane_kernel<FZ_SKM12, 64, 128, 2>);
+        case 32: return f(fz_tplane_kernel<FZ_SKM12, 32, 128, 2>);
+        }
+    if (prog == FZ_MFTA12) switch (s.rs) {
+        case 128: return f(fz_tplane_kernel<FZ_MFTA12, 128, 128, 2>);
+        case 96: return f(fz_tplane_kernel<FZ_MFTA12, 96, 96, 2>);
+        case 64: return f(fz_tplane_kernel<FZ_MFTA12, 64, 96, 2>);
+        }
     return cudaErrorInvalidConfiguration;
 }
-size_t tplane_smem(FzShape s) { return (prefetches(s.rs) ? 3 : 2) * (size_t)s.rs * s.rs * sizeof(float); }
+size_t tplane_smem(FzShape s) { return (s.ctas > 0 ? 3 : 2) * (size_t)s.rs * s.rs * sizeof(float); }
 
 }  // namespace
 
+// FZ_MFTA12, whose v is a second plane to wait for, always fetches ahead: CTAs that share an SM
+// walk over the planes.  FZ_SKM12 does where a plane is alone on its SM; three 96^2 planes
+// without a third buffer take 388 where two with one take 444.
 FzShape fz_tplane_shape(int prog, int N1, int N2) {
-    const int rs = N1;
-    if (N1 != N2 || N1 % 32 != 0 || (prog == FZ_MFTA12 && rs < 128)) return {};
-    return {rs == 128 ? 512 : rs == 96 ? 160 : rs == 64 ? 128 : 32, 0, rs};
+    if (N1 != N2) return {};
+    const bool w = prog == FZ_MFTA12;
+    switch (N1) {
+    case 128: return {512, 128, 128, 1};
+    case 96: return w ? FzShape{256, 96, 96, 2} : FzShape{160, 128, 96, 0};
+    case 64: return w ? FzShape{128, 96, 64, 4} : FzShape{64, 128, 64, 0};
+    case 32: return w ? FzShape{} : FzShape{32, 128, 32, 0};
+    }
+    return {};
 }
 
 cudaError_t prepare_tplane(int prog, FzShape s) {
@@ -486,12 +494,12 @@ cudaError_t launch_tplane(int prog, const FzParams<float>& p, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     return tplane_pick(prog, p.shape, [&](auto* k) {
         long long grid = p.njobs;
-        if (prefetches(p.shape.rs)) {
+        if (p.shape.ctas > 0) {
             int dev = 0, nsm = 0;
             cudaError_t r = cudaGetDevice(&dev);
             if (r == cudaSuccess) r = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
             if (r != cudaSuccess) return r;
-            grid = std::min(grid, (long long)nsm);
+            grid = std::min(grid, (long long)nsm * p.shape.ctas);
         }
         k<<<dim3((unsigned)grid), dim3(p.shape.threads), tplane_smem(p.shape), st>>>(q);
         count_launches(1);

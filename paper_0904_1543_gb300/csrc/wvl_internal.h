@@ -158,12 +158,13 @@ struct FzSeg {
     int RS;               // shared-memory row stride in elements
 };
 
-// Launch shape of a plane kernel (fz_plane_shape): threads, register cap, and the row length of
-// the transposing form's buffers (fused_plane.cu; 0: the general form).
+// Launch shape of a plane kernel (fz_plane_shape): threads, register cap, and of the transposing
+// form (fused_plane.cu) the side of its planes (0: the general form) and the CTAs per SM that
+// walk over the planes (0: a CTA per plane).
 struct FzShape {
-    int threads = 0, regs = 0, rs = 0;
+    int threads = 0, regs = 0, rs = 0, ctas = 0;
     bool operator!=(const FzShape& o) const {
-        return threads != o.threads || regs != o.regs || rs != o.rs;
+        return threads != o.threads || regs != o.regs || rs != o.rs || ctas != o.ctas;
     }
 };
 
