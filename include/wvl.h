@@ -243,10 +243,13 @@ wvl_status wvl_eloc_backward(const wvl_grid* grid, int prec, int norb,
  * wavelet transformation": the basis functions of Eq. wavef0 are
  * orthonormal, so <psi_i|psi_j> is the sum of the products of the
  * coefficients, taken on the compressed vectors).  Precision `prec` gives the
- * element type of a and b (float for WVL_F32, else double); every product is
- * formed in FP64 (an FP32 x FP32 product is exact there) and accumulated in
- * FP64 by a fixed-order two-stage reduction, so repeated calls give
- * identical results.
+ * element type of a and b (float for WVL_F32, else double).  Sums are
+ * accurate to FP64: wvl_overlap multiplies the digits of both sides exactly on
+ * the FP16 tensor cores and recombines them in integers and FP64 (each row on
+ * its own scale per slice of len; rows with an infinity or a NaN by FP64
+ * products); wvl_dot sums FP64 products, and FP32 products as exact pairs in
+ * compensated FP32 sums.  Orders are fixed, so repeated calls give identical
+ * results.
  *   wvl_overlap: S[i][j] = <a_i|b_j>, a: [na][len], b: [nb][len] (device),
  *     S: device double [na][nb], written.  When a == b and na == nb only the
  *     upper block triangle is computed and mirrored.

@@ -2,12 +2,12 @@
 //
 // A pass computes out(I) = sum_t f_t x(I - hl + off + t) on every line (the
 // 1D convolutions of Eqs. 1dconvtrans and kinetic1d).  For a tile of M = 128
-// lines and a window of N consecutive outputs (32 for the 16-tap filters,
-// 16 for the 29-tap kinetic filter) this is one small matrix product
-// D[line][j] = sum_k X[line][k] B[k][j] over the K = 48 input positions the
-// window reads, B being the banded filter matrix.  Both operands are turned into integers on a common
-// scale -- per line for X (its largest exponent), per filter for B -- and
-// split into S = 6 signed base-1024 digits:
+// lines and a window of N = 16 consecutive outputs this is one small matrix
+// product D[line][j] = sum_k X[line][k] B[k][j] over the K = 32 input positions
+// the window reads (48 for the 29-tap kinetic filter), B being the banded filter
+// matrix.  Both operands are turned into integers on a common scale -- per line for X
+// (its largest exponent, or that of its group of lines where the pass before handed its
+// integers over), per filter for B -- and split into S = 6 signed base-1024 digits:
 //
 //     X = sum_q x_q 1024^(S-q),  F = sum_p f_p 1024^(S-p),  |x_q|, |f_p| <= 512.
 //
