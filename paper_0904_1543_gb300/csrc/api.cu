@@ -113,6 +113,13 @@ struct Tune {
     bool persist = false;   // persistent double-buffered grid vs one CTA per job
 };
 
+// FP32 potential pass by rows: compensated density sums in shared memory, one float
+// pair per (output, line) of a tile
+template <typename T>
+static size_t pot_smem(int mode, int LT, int n) {
+    return (mode == M_POT && sizeof(T) == 4) ? (size_t)LT * n * 8 : 0;
+}
+
 // one staging buffer per CTA unless it prefetches (persistent grid, or the
 // orbital walk of the potential pass)
 static int nbuf(int mode, const Tune& t) { return (t.persist || mode == M_POT) ? 2 : 1; }
@@ -148,6 +155,16 @@ struct PassCall {
     bool emu = false;        // FP64 convolutions on the tensor cores (emu.cuh)
 };
 
+// output lines of a pass: length and number
+template <typename T>
+static void line_dims(const SegDesc<T>& d, int pass, int& n, int& N) {
+    pass_dims(d.Nf, pass, n, N);
+    if (d.gn > 0) {
+        n = d.gn;
+        N = d.gN;
+    }
+}
+
 // shared-memory row length of a staged line, in elements
 static int rowlen_of(int n, int R, const KindGeom& g, size_t elt) {
     int nch = (n + R - 1) / R;
@@ -169,18 +186,56 @@ static int rowlen_of(int n, int R, const KindGeom& g, size_t elt) {
     return rl;
 }
 
-// FP32 calls that pass32.cu takes: the potential pass, and the compressed passes where
-// every segment stores its whole grid.  The coefficients of a region or a box are looked up
-// one by one, which the row-wise kernel does better: 44 of 1037 us of H psi of 64 orbitals
-// on a ball in a coarse 48^3 cell.
+// FP32 calls that pass32.cu takes.  The compressed passes where every segment stores its
+// whole grid: the coefficients of a region or a box are looked up one by one, which the
+// row-wise kernel does better (44 of 1037 us of H psi of 64 orbitals on a ball in a coarse
+// 48^3 cell).  The potential pass from 5e5 output points on (1e5 without a density on the
+// orbitals' own grid): below, a CTA of one to three warps that computes 32 outputs per
+// thread leaves the SMs idle, and the row-wise kernel's four warps of shorter work are
+// faster.  Microseconds of the pass, row-wise and pass32.cu, with / without density: free 8^3
+// box (45^3 points), 2 orbitals 9.4, 11.1 / 6.5, 7.9; 4 orbitals 11.2, 13.0 / 7.6, 8.1; 8
+// orbitals 17.8, 16.3 / 10.9, 9.0; free 32^3, 8 orbitals 108, 52 / 56, 32; 64 orbitals
+// 453, 283 / 391, 211.  With a density lines of fewer than 32 outputs stay row-wise: a tile
+// has no full warp then (24 outputs, 64 orbitals: 31 against 36).
 template <typename T>
 static bool use_pass32(const PassCall<T>& c) {
     if (sizeof(T) != 4) return false;
-    if (c.mode == M_POT) return true;
+    if (c.mode == M_POT) {
+        long long points = 0, longer = 0;
+        bool plain = true;
+        for (const auto& d : c.segs) {
+            int n, N;
+            line_dims(d, c.pass, n, N);
+            const long long v = (long long)n * N * d.s.norb;
+            points += v;
+            if (d.user_rho == nullptr || n >= 32) longer += v;
+            plain = plain && d.user_rho == nullptr && d.s.vN1 == 0;
+        }
+        return points >= (plain ? 100000 : 500000) && 2 * longer >= points;
+    }
     if (c.mode != M_UNCOMP && c.mode != M_COMP) return false;
     for (const auto& d : c.segs)
         if (d.s.mapc != nullptr || d.s.bx1 != 0 || d.gn != 0) return false;
     return true;
+}
+
+// Orbitals per group of an FP32 potential pass of pass32.cu with a density, at most gmax
+// groups, `resident` CTAs at once.  A CTA's start and the flush of its density cost
+// about as much as three orbitals, so the group minimises waves x (orbitals + 3): 64 orbitals
+// on a free 16^3 box in 8 groups (one wave) 88 us, in 16 (1.5 waves) 116; 16 orbitals
+// 36 and 58.
+static int pass32_group(long long tiles, int norb, int gmax, long long resident) {
+    long long best = -1;
+    int opg = 1;
+    for (int g = (norb + gmax - 1) / gmax; g <= norb; ++g) {
+        const long long units = (norb + g - 1) / g * tiles;
+        const long long cost = (units + resident - 1) / resident * (g + 3);
+        if (best < 0 || cost < best) {
+            best = cost;
+            opg = g;
+        }
+    }
+    return opg;
 }
 
 template <typename T>
@@ -196,7 +251,8 @@ static bool tune_valid(const PassCall<T>& c, const Tune& t) {
             continue;
         }
         // the staging buffers must fit
-        if (nbuf(c.mode, t) * ((size_t)t.LT * rowlen_of(n, t.R, g, sizeof(T)) + 2) * sizeof(T) > 200 * 1024)
+        if (nbuf(c.mode, t) * ((size_t)t.LT * rowlen_of(n, t.R, g, sizeof(T)) + 2) * sizeof(T) +
+                pot_smem<T>(c.mode, t.LT, n) > 200 * 1024)
             return false;
         if (c.mode == M_POT && sizeof(T) == 8) {
             const int nslots = (NTHREADS / 32) * (32 / t.LT);
@@ -289,15 +345,26 @@ static wvl_status exec_call(PassCall<T>& c, const Tune& tn, cudaStream_t st) {
         int nmax = 0;
         int k = 0;
         const size_t first = i;
+        // pass32.cu's potential pass with a density: CTAs resident at once, and the
+        // orbital tiles of the launch, which share them
+        long long resident = 0, otiles = 0;
+        if (p32 && c.mode == M_POT) {
+            int nm = 0;
+            size_t sm = 0;
+            for (size_t j = i; j < c.segs.size() && j < i + MAXSEG; ++j) {
+                int n, N;
+                line_dims(c.segs[j], c.pass, n, N);
+                nm = std::max(nm, n);
+                sm = std::max(sm, pass32_smem(c.kind, c.mode, tn.LT, n, c.segs[j].user_rho != nullptr));
+                otiles += (long long)((N + tn.LT - 1) / tn.LT) * c.segs[j].s.norb;
+            }
+            resident = (long long)num_sms() * pass32_ctas(pass32_threads(tn.LT, nm), sm);
+        }
         for (; i < c.segs.size() && k < MAXSEG; ++i, ++k) {
             SegDesc<T>& d = c.segs[i];
             if (c.kind == K_KIN && i > first && d.hax != hax) break;
             Seg<T>& s = d.s;
-            pass_dims(d.Nf, c.pass, s.n, s.N);
-            if (d.gn > 0) {
-                s.n = d.gn;
-                s.N = d.gN;
-            }
+            line_dims(d, c.pass, s.n, s.N);
             if (emu) {
                 // units: 128-line tiles (the kernel walks their output windows)
                 s.nwin = (s.n + emu::window_n(c.kind) - 1) / emu::window_n(c.kind);
@@ -324,6 +391,9 @@ static wvl_status exec_call(PassCall<T>& c, const Tune& tn, cudaStream_t st) {
                 long long G = (want + s.tiles - 1) / s.tiles;
                 G = std::max(1LL, std::min<long long>(G, gmax));
                 s.opg = (int)((s.norb + G - 1) / G);
+                if (p32 && d.user_rho && gmax > 1)
+                    s.opg = pass32_group(s.tiles, s.norb, gmax,
+                                         std::max(1LL, resident * s.tiles * s.norb / otiles));
                 G = (s.norb + s.opg - 1) / s.opg;
                 d.groups = (int)G;
                 units = G;
@@ -385,7 +455,7 @@ static wvl_status exec_call(PassCall<T>& c, const Tune& tn, cudaStream_t st) {
         // two staging buffers, each rounded to 16 bytes
         const size_t per16 = 16 / sizeof(T);
         p.bufelems = (int)((smem + per16 - 1) / per16 * per16);
-        smem = nbuf(c.mode, tn) * (size_t)p.bufelems * sizeof(T);
+        smem = nbuf(c.mode, tn) * (size_t)p.bufelems * sizeof(T) + pot_smem<T>(c.mode, tn.LT, nmax);
         cudaError_t e = launch_pass<T>(c.kind, c.mode, tn.R, p, blk, smem, st, tn.persist);
         if (e != cudaSuccess) return cuda_fail(e, "pass launch");
     }

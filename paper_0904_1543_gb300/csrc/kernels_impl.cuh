@@ -61,8 +61,7 @@ static cudaError_t prepare_r() {
     if ((e = ensure_attr<T, K_SYN, M_PLAIN, R>()) != cudaSuccess) return e;
     if ((e = ensure_attr<T, K_ANA, M_COMP, R>()) != cudaSuccess) return e;
     if ((e = ensure_attr<T, K_ANA, M_PLAIN, R>()) != cudaSuccess) return e;
-    if constexpr (sizeof(T) == 8)   // (FP32: pass32.cu)
-        if ((e = ensure_attr<T, K_MF, M_POT, R>()) != cudaSuccess) return e;
+    if ((e = ensure_attr<T, K_MF, M_POT, R>()) != cudaSuccess) return e;
     if ((e = ensure_attr<T, K_MF, M_PLAIN, R>()) != cudaSuccess) return e;
     if ((e = ensure_attr<T, K_MFT, M_PLAIN, R>()) != cudaSuccess) return e;
     if ((e = ensure_attr<T, K_KIN, M_KMID, R>()) != cudaSuccess) return e;
@@ -82,8 +81,7 @@ static cudaError_t launch_r(int kind, int mode, const PassParams<T>& p, long lon
         if (mode == M_PLAIN) return launch_one<T, K_ANA, M_PLAIN, R>(p, nb, smem, st, ps);
         break;
     case K_MF:
-        if constexpr (sizeof(T) == 8)   // (FP32: pass32.cu)
-            if (mode == M_POT) return launch_one<T, K_MF, M_POT, R>(p, nb, smem, st, ps);
+        if (mode == M_POT) return launch_one<T, K_MF, M_POT, R>(p, nb, smem, st, ps);
         if (mode == M_PLAIN) return launch_one<T, K_MF, M_PLAIN, R>(p, nb, smem, st, ps);
         break;
     case K_MFT:

@@ -19,10 +19,12 @@
 // through shared memory.  The row-wise kernel copies them element by element, at two and
 // a half times the time of a plain pass.  The potential pass gains from 16-byte accesses to V
 // and its outputs and from shared memory for density sums only where there is a density
-// (a CTA without holds half as much, so twice as many fit).  Microseconds for 64 orbitals
+// (a CTA without holds half as much, so twice as many fit); an instance per kind of grid and
+// density keeps only its own state.  Microseconds for 64 orbitals
 // on a coarse 40^3 cell (32.8 M points, 39 at the copy rate), row-wise and here: synthesis
-// pass 1 140 / 102, analysis pass 3 138 / 90, potential pass without density 271 / 159;
-// 48 orbitals on 37x45x51: 139 / 104, 160 / 122, 379 / 170.  Plain and kinetic passes stay
+// pass 1 140 / 102, analysis pass 3 138 / 90; on 37x45x51 the potential pass takes 488 / 200
+// without a density and 568 / 268 with one, 48 orbitals there in the other two 139 / 104 and
+// 160 / 122.  Small calls stay with the row-wise kernel (use_pass32).  Plain and kinetic passes stay
 // with the row-wise kernel: 56 against 66, as its lines arrive by asynchronous copies while
 // other CTAs of the SM (fewer registers, more of them) compute.
 //
@@ -42,6 +44,11 @@ namespace {
 constexpr int P32_R = 8;          // outputs per thread and line
 constexpr int P32_THREADS = 256;  // most threads per CTA
 constexpr int P32_SMEM = 200 * 1024;
+// CTAs of the most threads that an SM's registers are split for: three (80 registers) in the
+// compressed passes; two (128) in the potential pass, which spills 404 bytes at 80 and whose
+// CTAs have 32 to 128 threads (64 orbitals with density on a free 16^3 box, in the same
+// groups: 172 us at 80, 116 at 128; on a periodic 37x45x51 cell 364 and 274)
+__host__ __device__ constexpr int p32_ctas(int mode) { return mode == M_POT ? 2 : 3; }
 
 template <typename F, int... I>
 __device__ __forceinline__ void p32_for_impl(F&& f, std::integer_sequence<int, I...>) {
@@ -219,8 +226,9 @@ __device__ __forceinline__ void stage_records(const Tile& t, const Seg<float>& S
     }
 }
 
-template <int KIND, int MODE>
-__global__ void __launch_bounds__(P32_THREADS, 3) pass32_kernel(const __grid_constant__ PassParams<float> p) {
+// VOWN: V and rho may live on another grid; RHO: there may be a density
+template <int KIND, int MODE, bool VOWN, bool RHO>
+__global__ void __launch_bounds__(P32_THREADS, p32_ctas(MODE)) pass32_kernel(const __grid_constant__ PassParams<float> p) {
     extern __shared__ __align__(16) float sm[];
     __shared__ double red[P32_THREADS / 32];
     constexpr int R = P32_R, HL = KT<KIND>::HL, NT = KT<KIND>::NT;
@@ -266,26 +274,22 @@ __global__ void __launch_bounds__(P32_THREADS, 3) pass32_kernel(const __grid_con
 
     // V and rho of output I of line l0 + k: (I + vo3) vplane + vl[k], the output's own index
     // unless they live on another grid (free lines)
-    long long vl[4] = {0, 0, 0, 0}, vplane = N;
-    int vo3 = 0, vn3 = 0x7fffffff;
-    const bool vown = MODE == M_POT && S.vN1 > 0;
-    if (MODE == M_POT) {
+    int vl[4] = {0, 0, 0, 0}, vplane = N, vo3 = 0, vn3 = 0x7fffffff;
+    const bool vown = VOWN && S.vN1 > 0;
+    if (vown) {
         #pragma unroll
-        for (int k = 0; k < 4; ++k) vl[k] = a + k;
-        if (vown) {
-            #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int X2 = (a + k) / S.N1, X1 = (a + k) - X2 * S.N1;
-                int w1 = X1 + S.vo1, w2 = X2 + S.vo2;
-                if (w1 >= S.vN1) w1 -= S.vN1;
-                if (w2 >= S.vN2) w2 -= S.vN2;
-                vl[k] = (long long)w2 * S.vN1 + w1;
-            }
-            vplane = (long long)S.vN1 * S.vN2;
-            vo3 = S.vo3;
-            vn3 = S.vN3;
+        for (int k = 0; k < 4; ++k) {
+            const int X2 = (a + k) / S.N1, X1 = (a + k) - X2 * S.N1;
+            int w1 = X1 + S.vo1, w2 = X2 + S.vo2;
+            if (w1 >= S.vN1) w1 -= S.vN1;
+            if (w2 >= S.vN2) w2 -= S.vN2;
+            vl[k] = w2 * S.vN1 + w1;
         }
+        vplane = S.vN1 * S.vN2;
+        vo3 = S.vo3;
+        vn3 = S.vN3;
     }
+    double* const rho_out = RHO ? S.rho : nullptr;
 
     #pragma unroll 1
     for (int orb = o0; orb < o1; ++orb) {
@@ -386,7 +390,7 @@ __global__ void __launch_bounds__(P32_THREADS, 3) pass32_kernel(const __grid_con
                         }
                         if (S.out) store4(S.out + oi, make_float4(y[0], y[1], y[2], y[3]), nv, vw);
                     }
-                    if (S.rho) {
+                    if (RHO && rho_out != nullptr) {
                         float4 h4 = make_float4(0.f, 0.f, 0.f, 0.f), w4 = h4;
                         float4* const ph = reinterpret_cast<float4*>(rhi + I * LT + l0);
                         float4* const pw = reinterpret_cast<float4*>(rlo + I * LT + l0);
@@ -455,7 +459,7 @@ __global__ void __launch_bounds__(P32_THREADS, 3) pass32_kernel(const __grid_con
     }
 
     // the group's density, consecutive lanes on consecutive lines
-    if (MODE == M_POT && S.rho != nullptr) {
+    if (RHO && rho_out != nullptr) {
         __syncthreads();
         const int l = threadIdx.x & (LT - 1);
         if (l >= t.lt) return;
@@ -467,7 +471,7 @@ __global__ void __launch_bounds__(P32_THREADS, 3) pass32_kernel(const __grid_con
             if (w2 >= S.vN2) w2 -= S.vN2;
             q0 = (long long)w2 * S.vN1 + w1;
         }
-        double* const rho = S.rho + (S.rho_gstride == 0 ? 0 : grp * S.rho_gstride) + q0;
+        double* const rho = rho_out + (S.rho_gstride == 0 ? 0 : grp * S.rho_gstride) + q0;
         #pragma unroll 2
         for (int I = threadIdx.x / LT; I < n; I += blockDim.x / LT) {
             int z = I + vo3;
@@ -479,7 +483,7 @@ __global__ void __launch_bounds__(P32_THREADS, 3) pass32_kernel(const __grid_con
     }
 }
 
-template <int KIND, int MODE>
+template <int KIND, int MODE, bool VOWN, bool RHO>
 cudaError_t p32_attr() {
     static std::atomic<unsigned long long> done{0};
     int dev = 0;
@@ -487,19 +491,25 @@ cudaError_t p32_attr() {
     if (err != cudaSuccess) return err;
     const unsigned long long bit = 1ull << (dev & 63);
     if (!(done.load() & bit)) {
-        err = cudaFuncSetAttribute(pass32_kernel<KIND, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, P32_SMEM);
+        err = cudaFuncSetAttribute((pass32_kernel<KIND, MODE, VOWN, RHO>), cudaFuncAttributeMaxDynamicSharedMemorySize, P32_SMEM);
         if (err != cudaSuccess) return err;
         done.fetch_or(bit);
     }
     return cudaSuccess;
 }
 
+// f(kind, mode, V and rho on another grid, density) of every instance
 template <typename F>
 void for_each_p32(F&& f) {
-#define P32_K(kind, mode) f(std::integral_constant<int, kind>{}, std::integral_constant<int, mode>{})
-    P32_K(K_SYN, M_UNCOMP);
-    P32_K(K_ANA, M_COMP);
-    P32_K(K_MF, M_POT);
+    using std::integral_constant;
+#define P32_K(kind, mode, vown, rho) \
+    f(integral_constant<int, kind>{}, integral_constant<int, mode>{}, std::vown##_type{}, std::rho##_type{})
+    P32_K(K_SYN, M_UNCOMP, false, false);
+    P32_K(K_ANA, M_COMP, false, false);
+    P32_K(K_MF, M_POT, false, false);
+    P32_K(K_MF, M_POT, false, true);
+    P32_K(K_MF, M_POT, true, false);
+    P32_K(K_MF, M_POT, true, true);
 #undef P32_K
 }
 
@@ -508,6 +518,10 @@ void for_each_p32(F&& f) {
 int pass32_threads(int LT, int nmax) {
     const int items = LT / 4 * ((nmax + P32_R - 1) / P32_R);
     return std::max(32, std::min((items + 31) / 32 * 32, P32_THREADS));
+}
+
+int pass32_ctas(int threads, size_t smem) {   // (1100: the static part)
+    return (int)std::max<size_t>(1, std::min<size_t>(227 * 1024 / (smem + 1100), 512 / threads));
 }
 
 size_t pass32_smem(int kind, int mode, int LT, int n, bool rho) {
@@ -524,11 +538,16 @@ cudaError_t launch_pass32(int kind, int mode, const PassParams<float>& p, long l
                           size_t smem, cudaStream_t st) {
     if (nunits <= 0) return cudaSuccess;
     if (nunits > 0x7fffffffLL || smem > (size_t)P32_SMEM) return cudaErrorInvalidConfiguration;
+    bool vown = false, rho = false;
+    for (int k = 0; k < p.nseg; ++k) {
+        vown |= mode == M_POT && p.seg[k].vN1 > 0;
+        rho |= mode == M_POT && p.seg[k].rho != nullptr;
+    }
     cudaError_t e = cudaErrorInvalidValue;
-    for_each_p32([&](auto k, auto m) {
-        if (kind != k() || mode != m()) return;
-        if ((e = p32_attr<k(), m()>()) != cudaSuccess) return;
-        pass32_kernel<k(), m()><<<dim3((unsigned)nunits), dim3(threads), smem, st>>>(p);
+    for_each_p32([&](auto k, auto m, auto v, auto r) {
+        if (kind != k() || mode != m() || vown != v() || rho != r()) return;
+        if ((e = p32_attr<k(), m(), v(), r()>()) != cudaSuccess) return;
+        pass32_kernel<k(), m(), v(), r()><<<dim3((unsigned)nunits), dim3(threads), smem, st>>>(p);
         count_launches(1);
         e = cudaGetLastError();
     });
@@ -537,8 +556,8 @@ cudaError_t launch_pass32(int kind, int mode, const PassParams<float>& p, long l
 
 cudaError_t prepare_pass32() {
     cudaError_t e = cudaSuccess;
-    for_each_p32([&](auto k, auto m) {
-        if (e == cudaSuccess) e = p32_attr<k(), m()>();
+    for_each_p32([&](auto k, auto m, auto v, auto r) {
+        if (e == cudaSuccess) e = p32_attr<k(), m(), v(), r()>();
     });
     return e;
 }

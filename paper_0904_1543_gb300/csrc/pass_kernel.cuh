@@ -443,15 +443,21 @@ pass_kernel(const __grid_constant__ PassParams<T> p) {
     const int slot = warp * spw + lane / LT;
     const int nslots = NWARPS * spw;
     constexpr bool KM = (MODE == M_KMID || MODE == M_KLAST);
-    // the potential pass (FP64 here; FP32: pass32.cu) keeps the density sums in registers
-    constexpr int CPT = MODE == M_POT ? POT_OUT / R : 1;
+    // FP32 potential pass: the density sums (compensated pairs) live in
+    // shared memory after the two staging buffers, slot [I][line] owned by
+    // the thread computing output I of that line, which keeps the kernel's
+    // registers (and so its occupancy) at the level of the plain passes; the
+    // FP64 pass keeps them in registers
+    constexpr bool RSM = (MODE == M_POT) && sizeof(T) == 4;
+    constexpr int CPT = (MODE == M_POT && !RSM) ? POT_OUT / R : 1;
+    float2* const rsm = reinterpret_cast<float2*>(smem_raw + 2 * (size_t)p.bufelems * sizeof(T));
 
     Job cur = make_job<T, MODE>(p, blockIdx.x);
     if (!cur.valid) return;
     stage<T, KIND, MODE>(p, cur, bufs);
     cp_commit();
 
-    RhoAcc<T> racc[CPT][R];   // M_POT: density per owned output
+    RhoAcc<T> racc[RSM ? 1 : CPT][RSM ? 1 : R];   // M_POT (FP64): density per owned output
     int b = 0;
 
     #pragma unroll 1
@@ -483,6 +489,8 @@ pass_kernel(const __grid_constant__ PassParams<T> p) {
         // M_COMP for the adjoint of E_loc: H psi scaled by 2 occ g
         T osc = T(1);
         if (MODE == M_COMP && S.gscale != nullptr) osc = T(2.0 * S.occ[orb] * S.gscale[0]);
+        // FP32 potential pass: the first orbital of the unit starts the sums
+        const bool first_orb = RSM && orb == (int)((cur.unit - S.blk0) / S.tiles) * S.opg;
         // index of output I of this line in V and rho: (I + vo3) vplane + vline,
         // the output's own index I N + a unless V and rho live on another grid
         // (free lines)
@@ -600,7 +608,16 @@ pass_kernel(const __grid_constant__ PassParams<T> p) {
                             if (S.out) S.out[obase + oidx] = y;
                             ech = fma(y, psi, ech);
                         }
-                        if (S.rho) racc[cc][r].add((T)occ * psi * psi);
+                        if (RSM) {
+                            if (S.rho) {
+                                float2& q = rsm[I * LT + line];
+                                FF f = first_orb ? FF{0.f, 0.f} : FF{q.x, q.y};
+                                ff_add(f, (float)occ * (float)psi * (float)psi);
+                                q = make_float2(f.hi, f.lo);
+                            }
+                        } else if (S.rho) {
+                            racc[RSM ? 0 : cc][RSM ? 0 : r].add((T)occ * psi * psi);
+                        }
                     }
                 }
                 if (MODE == M_KLAST || MODE == M_POT) e.add(ech);
@@ -614,7 +631,22 @@ pass_kernel(const __grid_constant__ PassParams<T> p) {
 
         // M_POT: the unit ends -> flush its density
         if (MODE == M_POT && (!nxt.valid || nxt.unit != cur.unit)) {
-            if (S.rho != nullptr && line_ok) {
+            if (RSM && S.rho != nullptr && line_ok) {
+                const long long grp = (cur.unit - S.blk0) / S.tiles;
+                #pragma unroll 1
+                for (int c = slot; c < nchunks; c += nslots)
+                    #pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const int I = c * R + r;
+                        if (I >= n) continue;
+                        const float2 q = rsm[I * LT + line];
+                        const double v = (double)q.x + (double)q.y;
+                        const long long oidx = vidx(I);
+                        if (S.rho_gstride == 0) S.rho[oidx] += v;
+                        else S.rho[grp * S.rho_gstride + oidx] = v;
+                    }
+            }
+            if (!RSM && S.rho != nullptr && line_ok) {
                 const long long grp = (cur.unit - S.blk0) / S.tiles;
                 #pragma unroll
                 for (int cc = 0; cc < CPT; ++cc) {
@@ -624,16 +656,17 @@ pass_kernel(const __grid_constant__ PassParams<T> p) {
                         const int I = c * R + r;
                         if (c < nchunks && I < n) {
                             const long long oidx = vidx(I);
-                            if (S.rho_gstride == 0) S.rho[oidx] += racc[cc][r].get();
-                            else S.rho[grp * S.rho_gstride + oidx] = racc[cc][r].get();
+                            if (S.rho_gstride == 0) S.rho[oidx] += racc[RSM ? 0 : cc][RSM ? 0 : r].get();
+                            else S.rho[grp * S.rho_gstride + oidx] = racc[RSM ? 0 : cc][RSM ? 0 : r].get();
                         }
                     }
                 }
             }
-            #pragma unroll
-            for (int cc = 0; cc < CPT; ++cc)
+            if (!RSM)
                 #pragma unroll
-                for (int r = 0; r < R; ++r) racc[cc][r].reset();
+                for (int cc = 0; cc < CPT; ++cc)
+                    #pragma unroll
+                    for (int r = 0; r < R; ++r) racc[RSM ? 0 : cc][RSM ? 0 : r].reset();
         }
 
         __syncthreads();   // buffer b is refilled by the next iteration's copies

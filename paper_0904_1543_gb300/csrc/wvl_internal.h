@@ -258,6 +258,7 @@ cudaError_t launch_pass(int kind, int mode, int R, const PassParams<T>& p,
 // The FP32 passes of pass32.cu: threads and shared memory of a launch whose longest
 // output line is n (rho: the potential pass has density sums), and the launch.
 int pass32_threads(int LT, int nmax);
+int pass32_ctas(int threads, size_t smem);   // potential pass: CTAs per SM
 size_t pass32_smem(int kind, int mode, int LT, int n, bool rho);
 cudaError_t launch_pass32(int kind, int mode, const PassParams<float>& p, long long nunits, int threads,
                           size_t smem, cudaStream_t st);
