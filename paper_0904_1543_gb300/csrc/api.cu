@@ -432,14 +432,6 @@ static wvl_status exec_call(PassCall<T>& c, const Tune& tn, cudaStream_t st) {
                                                       c.segs[first + q].Nf[2] / 2, s.norb, s.P, st);
                     if (e != cudaSuccess) return cuda_fail(e, "line exponent launch");
                 }
-            for (int q = 0; q < k; ++q) {
-                const Seg<T>& s = p.seg[q];
-                if (s.gin == nullptr) continue;
-                // (the exponents lie behind the scales of the two passes, build_calls)
-                const int* top = s.gmax + 3 * (s.norb * (s.P / 2));
-                cudaError_t e = launch_group_max(top, s.gmax, s.n, (long long)s.norb * (s.nsrc / s.n), st);
-                if (e != cudaSuccess) return cuda_fail(e, "line scale launch");
-            }
             cudaError_t e = launch_emu_t(c.kind, c.mode, p, blk, st);
             if (e == cudaErrorInvalidValue)
                 return fail(WVL_EUNSUPPORTED, "tensor-core pass: filter digit schedule not supported");
@@ -863,24 +855,28 @@ static std::vector<PassCall<T>> build_calls(int op, std::vector<CellRun<T>>& run
         break;
     }
     // Tensor-core passes of one operator hand integers with a scale per line to the next
-    // pass instead of FP64 numbers (emu_kernel.cu).  Scales and exponents lie in buffer C,
-    // free outside the kinetic passes: four arrays of at most P / 2 ints per orbital
-    // (the synthesis' line exponents, then the groups' largest exponents; the scales of
-    // passes 1 and 2; the lines' exponents).
+    // pass instead of FP64 numbers (emu_kernel.cu).  Their scales and exponents lie in buffer
+    // C, free outside the kinetic passes, per orbital: the exponents of the lines of passes 2
+    // and 3, the scales of pass 1, and the synthesis' line exponents, which the scales of
+    // pass 2 replace (at most P / 2 ints each).
     for (size_t i = 0; i + 1 < calls.size(); ++i) {
         PassCall<T>&c = calls[i], &d = calls[i + 1];
         if (!c.emu || c.kind == K_KIN || d.kind != c.kind || d.pass != c.pass + 1) continue;
         if (!emu_hands_over(c.kind)) continue;   // (never, for the filters of the method)
         for (size_t k = 0; k < runs.size(); ++k) {
-            int n, N;
-            pass_dims(runs[k].Nf, c.pass, n, N);
-            const long long slot = runs[k].norb * (runs[k].P / 2);
+            int n[4], N[4];
+            long long at[6] = {0};   // exponents of passes 2, 3; scales of 1; line exponents, scales of 2
+            for (int q = 1; q <= 3; ++q) pass_dims(runs[k].Nf, q, n[q], N[q]);
+            for (int q = 2; q <= 3; ++q)
+                at[q] = at[q - 1] + (long long)runs[k].norb * emu::hand_slots(n[q]) * N[q];
+            at[4] = at[3] + (long long)runs[k].norb * N[1];
             int* const g = reinterpret_cast<int*>(B(runs[k], C_));
-            c.segs[k].s.gout = g + c.pass * slot;
-            c.segs[k].s.gtop = g + 3 * slot;
-            d.segs[k].s.gin = g + c.pass * slot;
-            d.segs[k].s.gmax = g;
-            d.segs[k].s.nsrc = N;
+            Seg<T>&s = c.segs[k].s, &t = d.segs[k].s;
+            t.gmax = s.gtop = g + at[c.pass];
+            t.gin = s.gout = g + at[c.pass + 2];
+            if (s.lexp != nullptr) s.lexp = g + at[4];
+            s.nnext = n[d.pass];
+            t.nsrc = N[c.pass];
         }
     }
     return calls;

@@ -149,13 +149,25 @@ __host__ __device__ inline long long quantize(double x, int E) {
 constexpr long long DBIAS = 512LL * (1 + (1LL << 10) + (1LL << 20) + (1LL << 30) + (1LL << 40) + (1LL << 50));
 
 // X + DBIAS for X = round(t 2^(g + QBITS - E)), an integer t of scale 2^g (the output
-// of the pass before), |t| < 2^60, |t| 2^g <= 2^E, E - g >= HAND_MIN: one arithmetic shift
-// of 8 t, rounded half up
+// of the pass before), |t| < 2^60, |t| 2^g <= 2^E or t = 0: one arithmetic shift of 8 t, rounded half
+// up; to the left (exact) where the line's largest value is below the scale of t
 constexpr int HAND_MIN = QBITS - 2;
 __host__ __device__ inline long long requantize(long long t, int g, int E) {
     const int sh = E - HAND_MIN - g;
-    return ((t * 8 >> (sh > 63 ? 63 : sh)) + (2 * DBIAS + 1)) >> 1;
+    const long long u = (long long)((unsigned long long)t * 8 << (sh > 0 ? 0 : sh < -63 ? 63 : -sh));
+    return ((u >> (sh < 0 ? 0 : sh > 63 ? 63 : sh)) + (2 * DBIAS + 1)) >> 1;
 }
+
+// The largest exponents of the lines that a pass hands over to, without atomics: a line of n
+// elements crosses n neighbouring source lines (n divides their number), which at most
+// hand_slots(n) warps of 32 source lines share.  Each of these warps writes its own slot: the
+// warp of source line a that of its distance from the warp of the line's first one.
+__host__ __device__ inline int hand_slots(int n) {
+    return n % 32 == 0 ? n / 32 : 32 % n == 0 ? 1 : (n - 1) / 32 + 2;
+}
+// exponents below this one are as good as zero: the FP64 outputs of a line on this scale
+// keep a normal factor 2^(E + E_f - OUT_EXP)
+constexpr int HAND_FLOOR = -960;
 
 // signed base-1024 digits, most significant first: d[0] in [-512, 512],
 // the others in [-512, 511]
@@ -279,8 +291,6 @@ bool emu_hands_over(int kind);
 // P elements): lexp[orbital][x3 * 2 n2 + x2].
 cudaError_t launch_line_exp(const double* in, int* lexp, int n1, int n2, int n3, int norb,
                             long long P, cudaStream_t st);
-// largest of each group of n consecutive ints
-cudaError_t launch_group_max(const int* g, int* gmax, int n, long long ngroups, cudaStream_t st);
 // bounded waits of the emulated passes that ran out since the last call
 cudaError_t emu_take_timeouts(unsigned* count);
 // one bounded wait that cannot be satisfied, given up after about ms

@@ -22,18 +22,20 @@
 //      epilogue (transposed store, compressed scatter, V psi with density
 //      and Epot, kinetic K_p and Ekin).
 // Between the passes of one operator the outputs stay these integers, with a scale per
-// line (Seg::gout): the next pass shifts them to its own line's scale, the largest
-// exponent of the source lines that it crosses, without a scan of its inputs, and the FP64 pipe
-// (a conversion and a multiplication per output otherwise) is left out.  Where an FP64
-// array comes in, a line's exponent is the largest of a first read.
-// Every pass notes the largest magnitude of each line's integers, so that the scale of a
-// line is at most the spread inside its source lines above its own largest value; with the
-// bound |t| < 2^60 alone the error of H psi grew fourfold on coefficients that decay over
-// eleven decades.  It is now below that of FP64 hand-over: 1.2e-16 against
-// 1.5e-16 in the 2-norm (FP64 kernels 4.2e-16), 2.3e-16 against 2.7e-16 on decaying ones.
+// line (Seg::gout): the next pass shifts them to its own line's scale, the exponent of the
+// line's largest element, without a scan of its inputs, and the FP64 pipe
+// (a conversion and a multiplication per output otherwise) is left out.  The producing warps
+// note that exponent per line of the next pass as they store (warp_tops, emu.cuh: hand_slots).
+// Where an FP64 array comes in, a line's exponent is the largest of a first read.
+// One scale for all lines that cross the same source lines would do without the notes and
+// the shifts to the left (23.6 ms instead of 25.0 per headline step), but lines
+// far below their neighbours then lose their bits (a Gaussian of 2.5 points, modelled: at 1e-6
+// of its peak off two axes, 2e-12 of the element instead of 6e-15).  H psi of random coefficients:
+// 1.2e-16 in the 2-norm (FP64 kernels 4.2e-16).
 // Per headline step (192 orbitals): 30.9 ms with windows of 32 outputs, two CTAs per SM;
 // 29.2 with 16 outputs and three; 28.5 with fields masked and completed in one
-// operation; 24.7 with the integers and the copies (neither alone gains:
+// operation; 24.7 with the integers and the copies, 23.6 with the kinetic passes' rows,
+// 25.0 with a scale per line (integers and copies: neither alone gains,
 // without the scan's first read the slabs' loads wait for HBM, and copies of FP64 arrays leave
 // the scan; an L2 prefetch of the next slab gave 27.5, of the next tile 29.4, a
 // register prefetch of the next slab 31.7).
@@ -216,6 +218,41 @@ __device__ __forceinline__ void prefetch_epilogue(const Seg<double>& Sg, int o0,
     }
 }
 
+// Where a warp writes the largest exponents of its integer outputs, per output I and line of
+// the next pass (emu.cuh, hand_slots): source line a belongs to the next pass's line
+// I step + a / nnext, the warp's lines to more + 1 of them per output.
+struct HandOut {
+    int* top;    // output 0's entry of the first line, in the warp's slot of it
+    int* top0;   // the same entry in slot 0, which the others take
+    int step, more;
+};
+// position of the highest bit that differs from the sign; -1 for 0 and -1
+__device__ __forceinline__ int top_bit(int x) {
+    int p;
+    asm("bfind.s32 %0, %1;" : "=r"(p) : "r"(x));
+    return p;
+}
+// exponents as pairs of 16 bits, one pair per two outputs
+__device__ __forceinline__ unsigned pair16(int a, int b) { return __byte_perm((unsigned)a, (unsigned)b, 0x5410); }
+constexpr int HAND_NONE = -30000;
+// The largest over the warp's lanes of every one of the eight exponents in p, handed to
+// put(output, largest) by one lane each: half of the pairs go across in each of the first two
+// exchanges, so that six shuffles do (25.0 ms per headline step; 25.9 with eight warp
+// reductions and stores).
+template <typename F>
+__device__ __forceinline__ void warp_tops(const unsigned (&p)[4], F&& put) {
+    const int lane = threadIdx.x & 31;
+    const bool h = lane & 16, l = lane & 8;
+    unsigned q0 = h ? p[2] : p[0], q1 = h ? p[3] : p[1];
+    q0 = __vmaxs2(q0, __shfl_xor_sync(0xffffffffu, h ? p[0] : p[2], 16));
+    q1 = __vmaxs2(q1, __shfl_xor_sync(0xffffffffu, h ? p[1] : p[3], 16));
+    unsigned r = l ? q1 : q0;
+    r = __vmaxs2(r, __shfl_xor_sync(0xffffffffu, l ? q0 : q1, 8));
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) r = __vmaxs2(r, __shfl_xor_sync(0xffffffffu, r, o));
+    if ((lane & 7) < 2) put(2 * (lane >> 3) + (lane & 1), (lane & 1) ? (int)r >> 16 : (int)(short)r);
+}
+
 // one window's outputs of this thread (line er, outputs o0 .. o0 + N/2 - 1):
 // accumulators -> FP64 -> the pass's epilogue; returns the energy partial
 template <int KIND, int MODE, bool OUTI>
@@ -224,10 +261,11 @@ __device__ __forceinline__ double window_epilogue(const Seg<double>& Sg, uint32_
                                                   const double (&pa)[window_n(KIND) / 2],
                                                   const double (&pb)[window_n(KIND) / 2],
                                                   const double (&pc)[window_n(KIND) / 2],
-                                                  unsigned& top) {
+                                                  const HandOut* hos, const unsigned char* rowS) {
     constexpr int N = window_n(KIND), NH = N / 2;
     constexpr bool KM = (MODE == M_KMID || MODE == M_KLAST);
     const int n = Sg.n, NL = Sg.N;
+    const int gl = se;   // (integer output: the line's scale)
     se = max(-1022, min(1023, se));
     // 2^se as a double: the FP64 pipe is idle here, the integer pipes are not
     const double scale = __longlong_as_double((long long)(se + 1023) << 52);
@@ -267,7 +305,8 @@ __device__ __forceinline__ double window_epilogue(const Seg<double>& Sg, uint32_
         ce = (mu12 == 0 ? cc0 + cx : cc0 + Sg.ncoarse + 7LL * cx + mu12 - 1) + i2 * se_;
         co = cc0 + Sg.ncoarse + 7LL * cx + mu12 + 3 + i2 * so_;
     }
-    if (!row_ok) return 0.0;
+    if (OUTI ? lt <= (er & ~31) : !row_ok) return 0.0;   // (integer output: whole warps)
+    unsigned pe[NH / 2], nz = 0;   // exponents of the integer outputs; any of them not zero
     {
 #pragma unroll
         for (int c = 0; c < NH; ++c) {
@@ -285,13 +324,18 @@ __device__ __forceinline__ double window_epilogue(const Seg<double>& Sg, uint32_
             t = mad_wide(i[2], 1 << 20, t);
             t = mad_wide(i01, 1 << 30, t);
             const int I = o0 + c;
-            if (!full && I >= n) continue;
+            if (!full && I >= n) {
+                if (OUTI) pe[c / 2] = c & 1 ? pair16((int)pe[c / 2], HAND_NONE) : (unsigned)HAND_NONE;
+                continue;
+            }
             const long long oi = oi0 + (long long)c * NL;
             if constexpr (OUTI) {
-                // the next pass reads the integer and the line's scale
-                const int th = (int)(t >> 32);
-                top = max(top, (unsigned)(th ^ (th >> 31)));
-                reinterpret_cast<long long*>(Sg.out)[oi] = t;
+                // the next pass reads the integer, the line's scale and the largest exponent
+                // of its own lines
+                const int e = gl + 33 + top_bit((int)(t >> 32));
+                nz |= (unsigned)t | (unsigned)(t >> 32);
+                pe[c / 2] = c & 1 ? pair16((int)pe[c / 2], e) : (unsigned)e;
+                if (row_ok) reinterpret_cast<long long*>(Sg.out)[oi] = t;
                 continue;
             }
             const double val = (double)t * scale;
@@ -342,6 +386,44 @@ __device__ __forceinline__ double window_epilogue(const Seg<double>& Sg, uint32_
             }
         }
     }
+    if constexpr (OUTI) {
+        if (!row_ok || nz == 0)
+#pragma unroll
+            for (int k = 0; k < NH / 2; ++k) pe[k] = pair16(HAND_NONE, HAND_NONE);
+        // integers without a high word (zeros among them): the exact exponents
+        const unsigned small = __vmins2(__vmins2(pe[0], pe[1]), __vmins2(pe[2], pe[3]));
+        if (__any_sync(0xffffffffu, row_ok && nz != 0 && min((int)(short)small, (int)small >> 16) <= gl + 32)) {
+            int e[NH];
+#pragma unroll
+            for (int c = 0; c < NH; ++c) {
+                e[c] = HAND_NONE;
+                if (row_ok && o0 + c < n) {
+                    const long long t = reinterpret_cast<const long long*>(Sg.out)[oi0 + (long long)c * NL];
+                    if (t != 0) e[c] = gl + 64 - __clzll(t ^ (t >> 63));
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < NH / 2; ++k) pe[k] = pair16(e[2 * k], e[2 * k + 1]);
+        }
+        const HandOut ho = hos[er >> 5];
+        auto tops = [&](const unsigned (&m)[NH / 2], int* top) {
+            warp_tops(m, [&](int c, int e) {
+                if (o0 + c < n) top[(long long)(o0 + c) * ho.step] = e;
+            });
+        };
+        if (ho.more == 0) {
+            tops(pe, ho.top);
+        } else {   // the warp's lines belong to several of the next pass's
+            const int seg = rowS[er];
+#pragma unroll 1
+            for (int k = 0; k <= ho.more; ++k) {
+                unsigned m[NH / 2];
+#pragma unroll
+                for (int i = 0; i < NH / 2; ++i) m[i] = seg == k ? pe[i] : pair16(HAND_NONE, HAND_NONE);
+                tops(m, k == 0 ? ho.top : ho.top0 + k);
+            }
+        }
+    }
     return eacc;
 }
 
@@ -378,7 +460,8 @@ emu_pass_kernel(const __grid_constant__ Params ep) {
     __shared__ __align__(8) uint64_t mbar;
     __shared__ int rowE[M];
     __shared__ int rowG[INI ? M : 1];             // integer input: a line's first source line
-    __shared__ unsigned rowT[OUTI ? 2 * M : 1];   // integer output: largest magnitudes per line and half
+    __shared__ HandOut hos[OUTI ? M / 32 : 1];    // integer output
+    __shared__ unsigned char rowS[OUTI ? M : 1];  // a line's line of the next pass, from its warp's first
     __shared__ double red[WARPS];
 
     const PassParams<double>& p = ep.p;
@@ -497,13 +580,18 @@ emu_pass_kernel(const __grid_constant__ Params ep) {
             // ---------------------------- one exponent per line: given (synthesis
             // pass 1 on the full grid), or the whole line read, 8 lines in flight per warp
             if constexpr (INI) {
-                // the largest exponent of the n neighbouring source lines that this line
-                // crosses (n divides nsrc)
+                // the line's largest exponent, from the slots of the warps whose source lines
+                // it crosses (n divides nsrc)
                 if (tid < M) {
-                    const int ng = Sg.nsrc / n;
-                    const int k = (int)((unsigned)(J.a0 + tid) % (unsigned)ng);
-                    rowE[tid] = tid < J.lt ? Sg.gmax[(long long)J.orb * ng + k] : HAND_MIN;
-                    rowG[tid] = tid < J.lt ? k * n : 0;
+                    int e = HAND_FLOOR, a = 0;
+                    if (tid < J.lt) {
+                        a = (int)((unsigned)(J.a0 + tid) % (unsigned)(Sg.nsrc / n)) * n;
+                        const int ns = (a + n - 1) / 32 - a / 32 + 1;
+                        const int* g = Sg.gmax + (long long)J.orb * hand_slots(n) * Sg.N + J.a0 + tid;
+                        for (int k = 0; k < ns; ++k, g += Sg.N) e = max(e, *g);
+                    }
+                    rowE[tid] = e;
+                    rowG[tid] = a;
                 }
             } else if (MODE == M_UNCOMP && Sg.lexp != nullptr) {
                 for (int r = tid; r < M; r += THREADS)
@@ -598,7 +686,21 @@ emu_pass_kernel(const __grid_constant__ Params ep) {
                 if (++slot == NSLOT) slot = 0;
             };
             if constexpr (OUTI)
-                if (tid < J.lt) Sg.gout[(long long)J.orb * Sg.N + J.a0 + tid] = rowE[tid] + Ef - OUT_EXP;
+                if (tid < J.lt) {
+                    Sg.gout[(long long)J.orb * Sg.N + J.a0 + tid] = rowE[tid] + Ef - OUT_EXP;
+                    const int nn = Sg.nnext, w0 = J.a0 + (tid & ~31);   // the warp's first source line
+                    const int c0 = w0 / nn;
+                    rowS[tid] = (unsigned char)((J.a0 + tid) / nn - c0);
+                    if ((tid & 31) == 0) {
+                        HandOut h;
+                        h.step = Sg.N / nn;
+                        h.more = min(w0 + 31, Sg.N - 1) / nn - c0;
+                        const long long lines = (long long)n * h.step;   // of the next pass
+                        h.top0 = Sg.gtop + (long long)J.orb * hand_slots(nn) * lines + c0;
+                        h.top = h.top0 + (w0 / 32 - c0 * nn / 32) * lines;
+                        hos[tid >> 5] = h;
+                    }
+                }
             // kinetic passes: the thread of line er, outputs 8 half .. + 7 of a window, slices the
             // same positions of the line's slabs, and keeps them for the epilogue: the
             // outputs of window w are the positions of slab w + 1 (pa; pn is slab w + 2)
@@ -626,7 +728,6 @@ emu_pass_kernel(const __grid_constant__ Params ep) {
                 if (++slot == NSLOT) slot = 0;
             };
             double eacc = 0.0;
-            unsigned top = 0;   // largest high word of this thread's integer outputs' magnitudes
             int first = 0;   // slot of the window's first slab
 #pragma unroll 1
             for (int w = 0; w < nwin && !failed; ++w) {
@@ -669,7 +770,7 @@ emu_pass_kernel(const __grid_constant__ Params ep) {
                     break;
                 }
                 eacc += window_epilogue<KIND, MODE, OUTI>(Sg, tl, o + NH * half, er, J.lt, J.a0, J.orb,
-                                                    J.grp, rowE[er] + Ef - OUT_EXP, pa, pb, pc, top);
+                                                    J.grp, rowE[er] + Ef - OUT_EXP, pa, pb, pc, hos, rowS);
                 fence_before();
                 __syncthreads();   // accumulators are rewritten by the next window's MMAs
             }
@@ -679,15 +780,7 @@ emu_pass_kernel(const __grid_constant__ Params ep) {
                 if (tid == 0) Sg.part[(long long)J.orb * Sg.tiles + J.tt] = t;
                 __syncthreads();
             }
-            if constexpr (OUTI) rowT[half * M + er] = top;
             __syncthreads();   // rowE and the slab ring are reused by the next job
-            if constexpr (OUTI)
-                if (tid < J.lt) {
-                    // |t| <= 2^(32 + bits of the high word)
-                    const int bits = 64 - __clz((int)max(rowT[tid], rowT[M + tid]));
-                    const long long at = (long long)J.orb * Sg.N + J.a0 + tid;
-                    Sg.gtop[at] = Sg.gout[at] + max(HAND_MIN, bits);
-                }
             next_job(p, MODE, J);
         }
     }
@@ -827,26 +920,6 @@ __global__ void line_exp_kernel(const double* __restrict__ in, int* __restrict__
         const int v = lane == 0 ? m[0] : lane == 1 ? m[1] : lane == 2 ? m[2] : m[3];
         lexp[(long long)orb * N2 * N3 + (long long)(2 * i3 + a3) * N2 + 2 * i2 + a2] = v;
     }
-}
-
-// gmax[orbital][k] = the largest of g[orbital][k n .. k n + n - 1]; one warp each
-__global__ void group_max_kernel(const int* __restrict__ g, int* __restrict__ gmax, int n, long long ngroups) {
-    const long long k = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (k >= ngroups) return;
-    int e = -0x7fffffff;
-    for (int x = lane; x < n; x += 32) e = max(e, g[k * n + x]);
-    e = __reduce_max_sync(0xffffffffu, e);
-    if (lane == 0) gmax[k] = e;
-}
-
-cudaError_t launch_group_max(const int* g, int* gmax, int n, long long ngroups, cudaStream_t st) {
-    if (ngroups <= 0) return cudaSuccess;
-    const long long blocks = (ngroups + 7) / 8;
-    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    group_max_kernel<<<(unsigned)blocks, 256, 0, st>>>(g, gmax, n, ngroups);
-    count_launches(1);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_line_exp(const double* in, int* lexp, int n1, int n2, int n3, int norb,

@@ -64,11 +64,11 @@ struct Seg {
     const int* lexp;      // emulated M_UNCOMP: largest biased exponent of each input line,
                           //   [orbital][line] (null: the pass scans its lines)
     const int* gin;       // emulated passes: the input is integers, element e of scale
-                          //   2^gin[orbital][e mod nsrc] (null: FP64), and gmax[orbital][k] bounds
-    int* gmax;            //   the exponents of those of source lines k n .. k n + n - 1
-    int* gout;            // the output is integers, line a's of scale 2^gout[orbital][a] and
-    int* gtop;            //   with exponents up to gtop[orbital][a]
-    int nsrc;
+    const int* gmax;      //   2^gin[orbital][e mod nsrc] (null: FP64); gmax[orbital][slot][line]:
+                          //   exponents of each line's largest (emu::hand_slots)
+    int* gout;            // the output is integers, line a's of scale 2^gout[orbital][a], and
+    int* gtop;            //   gtop is gmax of the pass that reads them, on lines of nnext
+    int nsrc, nnext;
     long long clen;       // compressed length of one orbital (orbital stride there)
     long long ncoarse;    // scaling coefficients stored (start of the wavelet block)
     int bx1, bx2, bx3;    // free/surface boundary conditions: box extents inside the
