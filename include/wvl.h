@@ -244,10 +244,13 @@ wvl_status wvl_eloc_backward(const wvl_grid* grid, int prec, int norb,
  * orthonormal, so <psi_i|psi_j> is the sum of the products of the
  * coefficients, taken on the compressed vectors).  Precision `prec` gives the
  * element type of a and b (float for WVL_F32, else double).  Sums are
- * accurate to FP64: wvl_overlap multiplies the digits of both sides exactly on
- * the FP16 tensor cores and recombines them in integers and FP64 (each row on
- * its own scale per slice of len; rows with an infinity or a NaN by FP64
- * products); wvl_dot sums FP64 products, and FP32 products as exact pairs in
+ * accurate to FP64, the error of an entry below that of an FP64 sum of its
+ * products (of sum_k |a_k b_k|): wvl_overlap multiplies the digits of both sides
+ * exactly on the FP16 tensor cores and recombines them in integers and FP64
+ * (each row on its own scale per slice of len) where the magnitudes of the
+ * entry's own terms show that no more than min(len, 256) 2^-53 of their sum is
+ * lost, and sums FP64 products elsewhere and where there is an infinity or a
+ * NaN; wvl_dot sums FP64 products, and FP32 products as exact pairs in
  * compensated FP32 sums.  Orders are fixed, so repeated calls give identical
  * results.
  *   wvl_overlap: S[i][j] = <a_i|b_j>, a: [na][len], b: [nb][len] (device),
