@@ -260,7 +260,9 @@ wvl_status wvl_eloc_backward(const wvl_grid* grid, int prec, int norb,
  *     double[n], written.
  * len may be any compressed length (full grid 8 n1 n2 n3, or a region's
  * ncoarse + 7 nfine).  Workspace: wvl_overlap_workspace_size() (enough for
- * both calls with these sizes). */
+ * both calls with these sizes or smaller ones; wvl_dot of n rows needs that of
+ * na = n, nb = 1): about 16 bytes per entry and slice of len, in at most 32 MB or
+ * one slice. */
 wvl_status wvl_overlap_workspace_size(int prec, int na, int nb, long long len, size_t* bytes);
 wvl_status wvl_overlap(int prec, int na, const void* a, int nb, const void* b, long long len,
                        double* S, void* ws, size_t ws_bytes, void* stream);

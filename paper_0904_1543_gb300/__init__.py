@@ -397,7 +397,7 @@ def dot(a, b):
     n, ln = a2.shape
     d = torch.empty(n, dtype=torch.float64, device=a.device)
     prec = _prec(a)
-    ws, wsb, st = _overlap_ws(prec, n, n, ln, a.device)
+    ws, wsb, st = _overlap_ws(prec, n, 1, ln, a.device)
     _check(lib().wvl_dot(prec, n, a2.data_ptr(), b2.data_ptr(), ln, d.data_ptr(), ws, wsb, st))
     return d
 

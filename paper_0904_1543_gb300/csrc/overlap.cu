@@ -94,8 +94,7 @@ extern "C" wvl_status wvl_overlap_workspace_size(int prec, int na, int nb, long 
     if (na < 0 || nb < 0 || len < 0) return ov_fail(WVL_EINVAL, "negative size");
     const int a1 = std::max(na, 1), b1 = std::max(nb, 1);
     const long long l1 = std::max(len, 1LL);
-    size_t ov = overlap_mma_ws(a1, b1, l1, false);
-    if (a1 == b1) ov = std::max(ov, overlap_mma_ws(a1, b1, l1, true));
+    const size_t ov = overlap_mma_ws_bound(a1, b1, l1);
     const size_t dot = (size_t)std::max(na, 1) * DOT_BLOCKS * sizeof(double);
     *bytes = std::max(ov, dot);
     return WVL_OK;

@@ -79,6 +79,8 @@ static_assert(OM_P * OM_N <= 512 && OM_SMEM <= 227 * 1024, "tensor and shared me
 // the accuracy rule (om_exact_enough): an entry's error stays below OM_C 2^-53 sum |a_k b_k|
 constexpr int OM_C = 256;
 constexpr int OM_ZERO = -0x4000;          // exponent of a slice of zeros
+// most bytes of partials (or those of one slice)
+constexpr long long OM_PART = 32LL << 20;
 
 // an entry's sum over a slice: hi 2^32 + lo, hi from the diagonals 0..2; the sum of magnitudes
 struct __align__(16) OmPart {
@@ -698,20 +700,22 @@ __global__ void __launch_bounds__(256) overlap_sum_kernel(const OmParams q, doub
 
 // Slices of k: whole accumulations of OM_KC, as many as minimise the waves of
 // CTAs (one per SM) times a slice's length, each CTA costing about four
-// accumulations more (start, exponents, partials).  The same on every GPU, so that the
-// workspace bound holds.
+// accumulations more (start, exponents, partials), as long as their partials stay within
+// OM_PART (16 bytes per entry and slice: waves alone asked for 304 MB at 1000 vectors for
+// 4 %).  The same on every GPU, so that the workspace bound holds.
 // a slice's high integer takes 2^41 per accumulation
 long long om_min_slices(long long chunks) { return (chunks + (1 << 21) - 1) >> 21; }
-long long om_max_slices(long long len) {
+long long om_max_slices(int na, int nb, long long len) {
     const long long chunks = std::max(1LL, (len + OM_KC - 1) / OM_KC);
-    return std::max(om_min_slices(chunks), std::min(chunks, 2LL * OM_SLOTS));
+    const long long most = std::max(1LL, OM_PART / ((long long)sizeof(OmPart) * na * nb));
+    return std::max(om_min_slices(chunks), std::min({chunks, 2LL * OM_SLOTS, most}));
 }
 void om_shape(int na, int nb, long long len, bool sym, int& nsplit, long long& kper, long long& tiles) {
     const long long ti = (na + OM_M - 1) / OM_M, tj = (nb + OM_N - 1) / OM_N;
     tiles = sym ? ti * tj - ti * (ti - 1) : ti * tj;
     const long long chunks = std::max(1LL, (len + OM_KC - 1) / OM_KC);
     long long best = -1, ns = 1;
-    for (long long s = om_min_slices(chunks), e = om_max_slices(len); s <= e; ++s) {
+    for (long long s = om_min_slices(chunks), e = om_max_slices(na, nb, len); s <= e; ++s) {
         const long long cost = (tiles * s + OM_SLOTS - 1) / OM_SLOTS * ((chunks + s - 1) / s + 4);
         if (best < 0 || cost < best) {
             best = cost;
@@ -802,6 +806,16 @@ size_t overlap_mma_ws(int na, int nb, long long len, bool sym) {
     long long kper = 0, tiles = 0;
     om_shape(na, nb, len, sym, ns, kper, tiles);
     return om_bytes(na, nb, (size_t)na + (sym ? 0 : nb), ns, (size_t)ns * na * nb * sizeof(OmPart));
+}
+// Enough for every call of at most these sizes: grows with each of them (the slices of a call
+// do not: more rows, fewer slices)
+size_t overlap_mma_ws_bound(int na, int nb, long long len) {
+    const long long chunks = std::max(1LL, (len + OM_KC - 1) / OM_KC);
+    const long long ns = std::max(om_min_slices(chunks), std::min(chunks, 2LL * OM_SLOTS));
+    const size_t one = (size_t)na * nb * sizeof(OmPart);
+    const size_t parts = std::max(one * (size_t)om_min_slices(chunks),
+                                  std::min(one * (size_t)ns, std::max((size_t)OM_PART, one)));
+    return om_bytes(na, nb, (size_t)na + nb, ns, parts);
 }
 
 cudaError_t launch_overlap_mma(int prec, int na, const void* a, int nb, const void* b, long long len,

@@ -332,6 +332,7 @@ cudaError_t launch_reduce_parts_multi(const PartTasks& t, cudaStream_t st);
 // scalar products on the tensor cores (overlap_mma.cu): workspace bytes and launch;
 // bounded waits that ran out since the last call are added to *count
 size_t overlap_mma_ws(int na, int nb, long long len, bool sym);
+size_t overlap_mma_ws_bound(int na, int nb, long long len);   // of every call of at most these sizes
 cudaError_t launch_overlap_mma(int prec, int na, const void* a, int nb, const void* b, long long len,
                                bool sym, double* S, void* ws, cudaStream_t st);
 cudaError_t overlap_take_timeouts(unsigned* count);

@@ -6,6 +6,8 @@ with c = 600 from the arithmetic: the digits' error is kept below min(len, 256) 
 that sum by the accuracy rule (7 % more for its own rounding) or the entry is an FP64 sum
 (chains of at most 320 terms for these lengths), plus one FP64 addition per slice (at most
 304)."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -80,3 +82,41 @@ def test_lost_terms(G):
             a[0, 0], a[0, 1], b[0, 0], b[0, 1] = 1.0, 1e-10, 1e-10, 1.0
             ref = float(a[0, 0].double() * b[0, 0].double() + a[0, 1].double() * b[0, 1].double())
             assert abs(float(G.overlap(a, b)) / ref - 1.0) < 4e-16
+
+
+def _size(W, na, nb, length, prec):
+    need = ctypes.c_size_t(0)
+    assert W.lib().wvl_overlap_workspace_size(prec, na, nb, length, ctypes.byref(need)) == 0
+    return need.value
+
+
+def test_workspace_grows_with_every_size(W):
+    """A workspace for the largest block serves every smaller one; and its size is of the order of
+    the result's, not of the number of slices times it."""
+    for length in (1, 300, 20000, 884736, 40000000):
+        last = 0
+        for n in (1, 2, 31, 64, 200, 255, 256, 257, 300, 700, 1000, 1023, 1024, 1156, 2048, 4099, 8192):
+            s = _size(W, n, n, length, W.WVL_F32)
+            assert s >= last and s >= _size(W, n, 1, length, W.WVL_F32)
+            assert s >= _size(W, n, n, max(1, length // 3), W.WVL_F32)
+            last = s
+            if length <= 884736:
+                assert s <= 20 * n * n + (64 << 20), (n, s)
+
+
+@pytest.mark.gpu
+def test_workspace_of_the_largest_block(G):
+    import torch
+    lib, length = G.lib(), 5000
+    x = torch.rand((400, length), device="cuda") - 0.5
+    need = _size(G, 400, 400, length, G.WVL_F32)
+    ws = torch.empty(need, dtype=torch.uint8, device="cuda")
+    for n in (1, 3, 40, 129, 250, 311, 399, 400):
+        for m in (1, n):
+            S = torch.full((n, m), 7.0, dtype=torch.float64, device="cuda")
+            r = lib.wvl_overlap(G.WVL_F32, n, x.data_ptr(), m, x[1:].data_ptr() if n < 400 else x.data_ptr(),
+                                length, S.data_ptr(), ws.data_ptr(), need, None)
+            assert r == 0, (n, m)
+            y = (x[1:] if n < 400 else x)[:m]
+            torch.cuda.synchronize()
+            assert torch.allclose(S, x[:n].double() @ y.double().T, rtol=0, atol=1e-9)
