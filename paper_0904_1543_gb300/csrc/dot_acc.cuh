@@ -7,8 +7,8 @@
 // thread's sum keeps about 70 bits; FP64 begins with get().  Packed arithmetic,
 // two terms per lane and instruction.  The split needs products inside the
 // range of FP32: ok() is false where a term overflowed, is not finite, or
-// the largest is so small that the remainders may have underflowed, and the caller
-// then sums its terms in FP64.
+// the largest is so small that the remainders may have underflowed (zero among
+// them), and the caller then sums its terms on another scale or in FP64.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -51,8 +51,7 @@ template <> struct DotAcc<float> {
         const double lo = ((double)d.x + (double)d.y) + ((double)c.x + (double)c.y);
         return ((double)s.x + (double)s.y) + lo;
     }
-    // largest product in [2^-60, 2^100], or every term exactly zero; the sums finite
-    // (a NaN or an infinity shows in s)
+    // largest product in [2^-60, 2^100]; the sums finite (a NaN or an infinity shows in s)
     __device__ __forceinline__ bool ok() const {
         return (pmax >= 8.7e-19f && pmax <= 1.2e30f) && fabsf(s.x) < 1e35f && fabsf(s.y) < 1e35f;
     }

@@ -19,12 +19,49 @@
 namespace wvl {
 namespace {
 
+// FP32 terms (k = t0, t0 + step, ..) whose products left the range of the split (dot_acc.cuh),
+// or are all zero: once more on other scales, 2^96 up or down, and only what that does
+// not reach either in FP64 (a whole call on 256 rows of 884736 coefficients: 308 us in range,
+// 429 of 1e-12 and 421 of zeros, which straight to FP64 take 1366 and without the split 1269).
+// Inline and not unrolled, so that the kernel keeps five blocks per SM (three: 440 in range).
+__device__ __forceinline__ double dot_rescan(const float* x, const float* y, long long t0, long long end,
+                                          long long step, bool vec, bool up) {
+    const float2 sc = up ? make_float2(0x1p48f, 0x1p48f) : make_float2(0x1p-48f, 0x1p-48f);
+    DotAcc<float> acc;
+    float both = 0.f;   // largest of the terms' smaller factors: 0 if every term has a zero
+    auto add = [&](float2 u, float2 v) {
+        u = __fmul2_rn(u, sc);
+        v = __fmul2_rn(v, sc);
+        acc.add(u, v);
+        both = fmaxf(both, fmaxf(fminf(fabsf(u.x), fabsf(v.x)), fminf(fabsf(u.y), fabsf(v.y))));
+    };
+    if (vec) {
+        #pragma unroll 1
+        for (long long k = t0; k < end; k += step) {
+            const float4 u = __ldg(reinterpret_cast<const float4*>(x) + k);
+            const float4 v = __ldg(reinterpret_cast<const float4*>(y) + k);
+            add(make_float2(u.x, u.y), make_float2(v.x, v.y));
+            add(make_float2(u.z, u.w), make_float2(v.z, v.w));
+        }
+    } else {
+        #pragma unroll 1
+        for (long long k = t0; k < end; k += step) add(make_float2(x[k], 0.f), make_float2(y[k], 0.f));
+    }
+    if (acc.ok()) return acc.get() * (up ? 0x1p-96 : 0x1p96);
+    if (up && both == 0.f && acc.pmax == 0.f && isfinite(acc.s.x) && isfinite(acc.s.y)) return 0.0;
+    double s = 0.0;
+    const int per = vec ? 4 : 1;
+    for (long long k = t0; k < end; k += step)
+        for (int q = 0; q < per; ++q) s = fma((double)x[k * per + q], (double)y[k * per + q], s);
+    return s;
+}
+
 // d[o] partials: block b of orbital o sums a[o][k] b[o][k] over its k.  Rows of
 // whole 16-byte words are read as such (four of each row in flight); FP32 terms
 // are summed as in dot_acc.cuh (FP64 conversions and FMAs per term kept the FP64
 // pipe full: 1270 us for 256 orbitals of 884736 coefficients, 265 us now).
 template <typename T>
-__global__ void __launch_bounds__(256) dot_part_kernel(const T* __restrict__ a,
+__global__ void __launch_bounds__(256, 5) dot_part_kernel(const T* __restrict__ a,
                                                        const T* __restrict__ b, long long len,
                                                        double* __restrict__ part) {
     __shared__ double red[8];
@@ -56,12 +93,8 @@ __global__ void __launch_bounds__(256) dot_part_kernel(const T* __restrict__ a,
         for (long long k = t0; k < len; k += step) acc.add(x[k], y[k]);
     }
     double s = acc.get();
-    if (!acc.ok()) {
-        s = 0.0;
-        const int per = vec ? PER : 1;
-        for (long long k = t0; k < len / per; k += step)
-            for (int q = 0; q < per; ++q) s = fma((double)x[k * per + q], (double)y[k * per + q], s);
-    }
+    if constexpr (sizeof(T) == 4)
+        if (!acc.ok()) s = dot_rescan(x, y, t0, vec ? len / PER : len, step, vec, acc.pmax < 1.f);
     #pragma unroll
     for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
