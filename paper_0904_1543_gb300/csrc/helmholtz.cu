@@ -35,6 +35,7 @@
 
 #include <cuda_runtime.h>
 
+#include "dot_acc.cuh"
 #include "wvl_internal.h"
 
 namespace wvl {
@@ -116,58 +117,42 @@ __device__ __forceinline__ void hz_minv(const HzParams& h, int o, float* minv) {
     if (threadIdx.x < 8) minv[threadIdx.x] = (float)(1.0 / (h.diag[threadIdx.x] - h.eps[o]));
 }
 
-// Scalar-product terms of a thread: each product split into its FP32 value and FMA
-// remainder, summed as a compensated pair (two-sum, about 48 bits), two at a
-// time; FP64 from the warp on (per thread, the conversions and additions kept
-// hz_col's FP64 pipe busy for a third of its time).  The quotients these sums
-// enter, alpha and beta, are FP32 numbers.
-struct HzDot {
-    float2 s{0.f, 0.f}, c{0.f, 0.f};
-    float pmax = 0.f;
-    __device__ __forceinline__ void add(float2 x, float2 y) {
-        const float2 m1 = make_float2(-1.f, -1.f);
-        const float2 p = __fmul2_rn(x, y);
-        const float2 e = __ffma2_rn(x, y, make_float2(-p.x, -p.y));
-        const float2 t = __fadd2_rn(s, p);
-        const float2 b = __ffma2_rn(s, m1, t);       // t - s
-        const float2 r = __ffma2_rn(b, m1, t);       // t - b
-        const float2 e1 = __ffma2_rn(r, m1, s);      // s - (t - b)
-        const float2 e2 = __ffma2_rn(b, m1, p);      // p - b
-        s = t;
-        c = __fadd2_rn(c, __fadd2_rn(e, __fadd2_rn(e1, e2)));
-        pmax = fmaxf(pmax, fmaxf(fabsf(p.x), fabsf(p.y)));
-    }
-    // the products inside the range in which the split is exact (dot_acc.cuh)
-    __device__ __forceinline__ bool ok() const {
-        return pmax >= 8.7e-19f && pmax <= 1.2e30f && fabsf(s.x) < 1e35f && fabsf(s.y) < 1e35f;
-    }
-};
-// a += x, the rounding error of hi into lo
-__device__ __forceinline__ void hz_pair_add(float& hi, float& lo, float xh, float xl) {
-    const float t = hi + xh, b = t - hi;
-    lo += ((hi - (t - b)) + (xh - b)) + xl;
-    hi = t;
+// The block's total of the threads' scalar-product terms (dot_acc.cuh: three FP32 numbers of
+// about 70 bits), in a fixed order; FP64 from the warp on (per thread, the conversions and
+// additions kept hz_col's FP64 pipe busy for a third of its time).  wide: the FP64 sum of a
+// thread whose terms left the range of the split.
+__device__ __forceinline__ float hz_two_sum(float& a, float x) {
+    const float t = a + x, b = t - a, e = (a - (t - b)) + (x - b);
+    a = t;
+    return e;
 }
-
-// the block's total in a fixed order; wide: the FP64 sum of a thread whose terms left
-// the range of the split
-__device__ __forceinline__ double hz_block_sum(const HzDot& d, bool on, bool ok, double wide, double* red) {
-    float hi = on && ok ? d.s.x : 0.f, lo = on && ok ? d.c.x : 0.f;
-    if (on && ok) hz_pair_add(hi, lo, d.s.y, d.c.y);
+__device__ __forceinline__ void hz_add3(float (&v)[3], float h, float m, float l) {
+    const float e = hz_two_sum(v[0], h);
+    const float e1 = hz_two_sum(v[1], m), e2 = hz_two_sum(v[1], e);
+    v[2] += l + (e1 + e2);
+}
+__device__ __forceinline__ double hz_block_sum(const DotAcc<float>& d, bool on, bool ok, double wide, double* red) {
+    float v[3] = {0.f, 0.f, 0.f};
+    if (on && ok) {
+        v[0] = d.s.x;
+        v[1] = d.c.x;
+        v[2] = d.d.x;
+        hz_add3(v, d.s.y, d.c.y, d.d.y);
+    }
     #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        const float xh = __shfl_down_sync(0xffffffffu, hi, o), xl = __shfl_down_sync(0xffffffffu, lo, o);
-        hz_pair_add(hi, lo, xh, xl);
+        const float h = __shfl_down_sync(0xffffffffu, v[0], o), m = __shfl_down_sync(0xffffffffu, v[1], o);
+        hz_add3(v, h, m, __shfl_down_sync(0xffffffffu, v[2], o));
     }
-    double v = (double)hi + (double)lo;
+    double t = (double)v[0] + ((double)v[1] + (double)v[2]);
     if (__any_sync(0xffffffffu, on && !ok)) {
         #pragma unroll
         for (int o = 16; o > 0; o >>= 1) wide += __shfl_down_sync(0xffffffffu, wide, o);
-        v += wide;
+        t += wide;
     }
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
     __syncthreads();
-    double t = 0.0;
+    t = 0.0;
     if (threadIdx.x == 0)
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
     return t;
@@ -194,7 +179,7 @@ __global__ void __launch_bounds__(256) hz_init_kernel(const __grid_constant__ Hz
     const int n1 = h.N1 / 2, n2 = h.N2 / 2, m = (int)(h.P / 8);
     const float* const gc = h.g + (long long)o * h.P;
     float* const r = h.r + (long long)o * h.P;
-    HzDot acc;
+    DotAcc<float> acc;
     for (int k = blockIdx.x * 256 + threadIdx.x; k < m; k += gridDim.x * 256) {
         const int row = k / n1, i1 = k - row * n1;
         const int i3 = row / n2, i2 = row - i3 * n2;
@@ -336,7 +321,7 @@ __global__ void hz_col_kernel(const __grid_constant__ HzParams h) {
     __syncthreads();
     double s = 0.0;
     bool ok = true;
-    HzDot dot;
+    DotAcc<float> dot;
     if (on) {
         hz_col_sum(X + 4 * cv, rowoff + HZ_PAD + r0 - HZ_LO, h.tap[2], acc);
         #pragma unroll
@@ -373,7 +358,7 @@ __global__ void __launch_bounds__(256) hz_step_kernel(const __grid_constant__ Hz
     __syncthreads();
     float4* const r4 = reinterpret_cast<float4*>(h.r + (long long)o * h.P);
     const float4* const q4 = reinterpret_cast<const float4*>(h.q + (long long)o * h.P);
-    HzDot acc;
+    DotAcc<float> acc;
     #pragma unroll 4
     for (int v = blockIdx.x * 256 + threadIdx.x; v < nv; v += gridDim.x * 256) {
         const int mu = hz_mu(v, ncv, h.N2);
