@@ -11,15 +11,17 @@
 // of a packed FMA as they are loaded; a row item has to copy each value into both
 // halves.  Extents are compile-time constants, which leaves one XOR per 16-byte load of address
 // arithmetic.  Microseconds of SYN3 + SKM12 / MFTA12 in the general form and here: 128^2 (48
-// orbitals) 812 / 432 and 688 / 330 (746 / 388 with extents from memory), 96^2 (64) 456 /
-// 219 and 388 / 207, 64^2 (128) 267 / 123 and 239 / 119, 32^2 (512) 150 / 78 and 125 / 78 (so
+// orbitals) 812 / 432 and 688 / 324 (746 / 388 with extents from memory), 96^2 (64) 456 /
+// 219 and 388 / 209, 64^2 (128) 267 / 123 and 239 / 119, 32^2 (512) 150 / 78 and 125 / 78 (so
 // MFTA12 keeps the general form there).  Also tried at 128^2, with extents from memory: items of
 // four lines (256 threads: 760 / 447), T_2 as items along the contiguous axis of a transposed s
 // (800 to 820), a warp of its own for the copies (1153 / 1205: one warp's copies in flight
 // are too few).
 //
-// The outputs' sums keep the order of the general form except MFT_1 and MFT_2, whose order
-// is exchanged; t and Ekin are the same bits.
+// All sums keep the order of the general form, so that an orbital's results do not depend on
+// the number of planes in its call, which chooses the form (fz_plane_shape): the same bits.
+// MFT_1 before MFT_2 therefore, by rows and without a transpose (128^2 324 us, with MFT_2
+// first, both as line items, 331; 96^2 209 and 207).
 #include <algorithm>
 #include <type_traits>
 
@@ -389,30 +391,35 @@ __global__ void __maxnreg__(REGS) fz_tplane_kernel(const __grid_constant__ FzTil
         } else {
             cp_wait<1>();      // x; v may still be under way
             __syncthreads();
-            // w = MFT_1 MFT_2 x + v -> X as [I2][I1]
-            w2.each([&](int kb, int u) {
-                line_item<K_MFT, RS, LP>(X, kb, nb2, u, p.td[0], acc);
-                store_trans<RS, LP>(Y, kb, u, acc);
+            // w = MFT_2 MFT_1 x + v -> X, MFT_1 first as in the general form
+            const int nch = N1 / 16;
+            const Walk wr(warp, nw, nch, N2 / 32);   // a lane per I2, chunks of 16
+            wr.each([&](int ch, int rb) {
+                const int row = rb * 32 + lane;
+                float win[4 * RowWin<K_MFT>::WV], v[16];
+                row_win<K_MFT, RS>(X, row, ch, nch, win);
+                row_fir<K_MFT, RowWin<K_MFT>::D>(win, p.tp[1], v);
+                store_chunk<RS>(Y, row, ch, v);
             });
             cp_wait<0>();
             __syncthreads();
-            w1.each([&](int kb, int u) {
-                line_item<K_MFT, RS, LP>(Y, kb, nb1, u, p.td[0], acc);
-                const unsigned bx = trans_base<RS, LP>(X, kb, u), bz = trans_base<RS, LP>(Z, kb, u);
+            w2.each([&](int kb, int u) {
+                line_item<K_MFT, RS, LP>(Y, kb, nb2, u, p.td[0], acc);
                 #pragma unroll
-                for (int e = 0; e < LP; ++e)
+                for (int h = 0; h < 2; ++h) {
+                    const unsigned o = (2 * kb + h) * 8 * PlaneBuf<RS>::ROW + line_off<LP>(u, 2 * kb + h);
                     #pragma unroll
-                    for (int h = 0; h < 4; ++h) {
-                        const float4 v = trans_word<RS>(bz, e, h), m = line_word<LP>(acc, e, h);
-                        trans_word<RS>(bx, e, h) = make_float4(m.x + v.x, m.y + v.y, m.z + v.z, m.w + v.w);
+                    for (int k = 0; k < 8; ++k) {
+                        const float2 v = half_word(((Z + o) ^ (k << 4)) + k * PlaneBuf<RS>::ROW);
+                        half_word(((X + o) ^ (k << 4)) + k * PlaneBuf<RS>::ROW) =
+                            make_float2(acc[8 * h + k][0].x + v.x, acc[8 * h + k][0].y + v.y);
                     }
+                }
             });
             __syncthreads();
             if (more) fetch_plane<RS>(Z, nx.S->in + nx.base);
             cp_commit();
-            // w' = A_2 A_1 w, A_1 with a lane per I2, chunks of 16
-            const int nch = N1 / 16;
-            const Walk wr(warp, nw, nch, N2 / 32);
+            // w' = A_2 A_1 w
             wr.each([&](int ch, int rb) {
                 const int row = rb * 32 + lane;
                 float win[4 * RowWin<K_ANA>::WV], v[16];
@@ -486,6 +493,7 @@ cudaError_t launch_tplane(int prog, const FzParams<float>& p, cudaStream_t st) {
         tap_pairs<K_MF>(p.tap[3], q.tp[1]);
     } else {
         tap_pairs<K_ANA>(p.tap[1], q.tp[0]);
+        tap_pairs<K_MFT>(p.tap[0], q.tp[1]);
     }
     q.njobs = p.njobs;
     q.nseg = p.nseg;
