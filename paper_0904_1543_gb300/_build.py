@@ -21,7 +21,8 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CU_SOURCES = ["api.cu", "kernels_f64.cu", "kernels_f32.cu", "pass32.cu", "fused_plane.cu", "emu_kernel.cu", "fused_kernel.cu",
               "reduce.cu", "noalloc.cu", "pcg.cu", "probe.cu", "overlap.cu", "overlap_mma.cu", "helmholtz.cu"]
 CPP_SOURCES = ["filters.cpp"]
-HEADERS = ["wvl_internal.h", "taps.h", "pass_kernel.cuh", "kernels_impl.cuh", "emu.cuh", "fused.cuh", "tcgen05.cuh", "dot_acc.cuh"]
+HEADERS = ["wvl_internal.h", "taps.h", "pass_kernel.cuh", "kernels_impl.cuh", "emu.cuh", "fused.cuh", "tcgen05.cuh", "dot_acc.cuh",
+           "static_for.cuh"]
 
 
 def nvcc() -> str:

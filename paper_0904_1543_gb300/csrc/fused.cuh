@@ -1,24 +1,12 @@
 // Shared by the fused chain's kernels (fused_kernel.cu, fused_plane.cu).
 #pragma once
-#include <utility>
-
 #include <cuda_runtime.h>
 
 #include "pass_kernel.cuh"
+#include "static_for.cuh"
 
 namespace wvl {
 namespace {
-
-// compile-time loop: f(integral_constant<int, 0>) ... f(integral_constant<int, N - 1>),
-// so tap indices are constants by construction (no run-time index or test)
-template <typename F, int... I>
-__device__ __forceinline__ void static_for_impl(F&& f, std::integer_sequence<int, I...>) {
-    (f(std::integral_constant<int, I>{}), ...);
-}
-template <int N, typename F>
-__device__ __forceinline__ void static_for(F&& f) {
-    static_for_impl(f, std::make_integer_sequence<int, N>{});
-}
 
 // Energy accumulator of an energy partial (one CTA's share of Ekin): FP64
 // in the FP64 form; in the FP32 form a compensated FP32 pair (two-sum,

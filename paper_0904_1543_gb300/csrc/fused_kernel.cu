@@ -876,7 +876,6 @@ cudaError_t fz_launch(const FzParams<T>& p, size_t smem, cudaStream_t st) {
                 tap_pairs<K_ANA>(q.tap[1], q.tp[1]);
             }
             if (s.regs == 96) return fz_plane_launch<T, PROG, 96>(q, s.threads, smem, st);
-            if (s.regs == 112) return fz_plane_launch<T, PROG, 112>(q, s.threads, smem, st);
             return fz_plane_launch<T, PROG, 128>(q, s.threads, smem, st);
         } else {
             return fz_plane_launch<T, PROG, 255>(p, s.threads, smem, st);
@@ -929,10 +928,8 @@ cudaError_t prepare_fused_kernels() {
         return fz_ensure_attr<T, FZ_MFTA12, 255>();
     } else {
         if ((e = fz_ensure_attr<T, FZ_SKM12, 96>()) != cudaSuccess) return e;
-        if ((e = fz_ensure_attr<T, FZ_SKM12, 112>()) != cudaSuccess) return e;
         if ((e = fz_ensure_attr<T, FZ_SKM12, 128>()) != cudaSuccess) return e;
         if ((e = fz_ensure_attr<T, FZ_MFTA12, 96>()) != cudaSuccess) return e;
-        if ((e = fz_ensure_attr<T, FZ_MFTA12, 112>()) != cudaSuccess) return e;
         if ((e = fz_ensure_attr<T, FZ_MFTA12, 128>()) != cudaSuccess) return e;
         for (int rs = 32; rs <= 128; rs += 32)
             for (int prog : {FZ_SKM12, FZ_MFTA12}) {

@@ -23,6 +23,7 @@
 // MFT_1 before MFT_2 therefore, by rows and without a transpose (128^2 324 us, with MFT_2
 // first, both as line items, 331; 96^2 209 and 207).
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "fused.cuh"
@@ -103,44 +104,36 @@ __device__ __forceinline__ void line_item(unsigned buf, int kb, int nb, int u, c
         });
     });
 }
-// the item's outputs, transposed: line LP u + e becomes a row, its words 4 kb + h
-template <int RS, int LP>
+// the item's outputs, transposed: line 2 u + e becomes a row, its words 4 kb + h
+template <int RS>
 __device__ __forceinline__ unsigned trans_base(unsigned buf, int kb, int u) {
-    const int s = LP == 4 ? (4 * (u & 1)) ^ ((u >> 1) & 3) : (2 * (u & 3)) ^ ((u >> 2) & 3);
-    return buf + LP * u * PlaneBuf<RS>::ROW + ((unsigned)((4 * kb) ^ s) << 4);
+    const int s = (2 * (u & 3)) ^ ((u >> 2) & 3);
+    return buf + 2 * u * PlaneBuf<RS>::ROW + ((unsigned)((4 * kb) ^ s) << 4);
 }
 template <int RS>
 __device__ __forceinline__ float4& trans_word(unsigned base, int e, int h) {
     return word((base ^ ((e ^ h) << 4)) + e * PlaneBuf<RS>::ROW);
 }
 // outputs 4 h .. 4 h + 3 of line e
-template <int LP>
-__device__ __forceinline__ float4 line_word(const float2 (&acc)[16][LP / 2], int e, int h) {
+__device__ __forceinline__ float4 line_word(const float2 (&acc)[16][1], int e, int h) {
     float q[4];
     #pragma unroll
-    for (int k = 0; k < 4; ++k) q[k] = (e & 1) ? acc[4 * h + k][e / 2].y : acc[4 * h + k][e / 2].x;
+    for (int k = 0; k < 4; ++k) q[k] = e ? acc[4 * h + k][0].y : acc[4 * h + k][0].x;
     return make_float4(q[0], q[1], q[2], q[3]);
 }
-template <int RS, int LP>
-__device__ __forceinline__ void store_trans(unsigned buf, int kb, int u, const float2 (&acc)[16][LP / 2]) {
-    const unsigned base = trans_base<RS, LP>(buf, kb, u);
+template <int RS>
+__device__ __forceinline__ void store_trans(unsigned buf, int kb, int u, const float2 (&acc)[16][1]) {
+    const unsigned base = trans_base<RS>(buf, kb, u);
     #pragma unroll
-    for (int e = 0; e < LP; ++e)
+    for (int e = 0; e < 2; ++e)
         #pragma unroll
-        for (int h = 0; h < 4; ++h) trans_word<RS>(base, e, h) = line_word<LP>(acc, e, h);
+        for (int h = 0; h < 4; ++h) trans_word<RS>(base, e, h) = line_word(acc, e, h);
 }
 // the item's outputs to the global plane of N columns at g
-template <int LP>
-__device__ __forceinline__ void store_global(float* g, int N, int kb, int u, const float2 (&acc)[16][LP / 2]) {
-    g += (long long)(16 * kb) * N + LP * u;
+__device__ __forceinline__ void store_global(float* g, int N, int kb, int u, const float2 (&acc)[16][1]) {
+    g += (long long)(16 * kb) * N + 2 * u;
     #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        if constexpr (LP == 4)
-            *reinterpret_cast<float4*>(g + (long long)k * N) =
-                make_float4(acc[k][0].x, acc[k][0].y, acc[k][LP / 2 - 1].x, acc[k][LP / 2 - 1].y);
-        else
-            *reinterpret_cast<float2*>(g + (long long)k * N) = acc[k][0];
-    }
+    for (int k = 0; k < 16; ++k) *reinterpret_cast<float2*>(g + (long long)k * N) = acc[k][0];
 }
 // word i (0 to 3) of chunk a (16 columns) of row: (chunk_base(row, a) ^ (i << 4))
 template <int RS>
@@ -243,7 +236,7 @@ struct Walk {
     }
 };
 
-template <int PROG, int RS, int REGS, int LP>
+template <int PROG, int RS, int REGS>
 __global__ void __maxnreg__(REGS) fz_tplane_kernel(const __grid_constant__ FzTileParams p) {
     __shared__ double red[FZ_PTHREADS / 32];
     unsigned X = 0, Z = 2 * PlaneBuf<RS>::SIZE;
@@ -264,11 +257,11 @@ __global__ void __maxnreg__(REGS) fz_tplane_kernel(const __grid_constant__ FzTil
         const FzSeg<float>& S = *c.S;
         // items along axis 2 ([I2][I1] planes) and along axis 1 ([I1][I2])
         const int nb2 = N2 / 8, nb1 = N1 / 8;
-        const Walk w2(threadIdx.x, T, N2 / 16, N1 / LP), w1(threadIdx.x, T, N1 / 16, N2 / LP);
+        const Walk w2(threadIdx.x, T, N2 / 16, N1 / 2), w1(threadIdx.x, T, N1 / 16, N2 / 2);
         const bool more = job + gridDim.x < p.njobs;
         Plane nx = c;
         if (more) nx = plane_of(p, job + gridDim.x);
-        float2 acc[16][LP / 2];
+        float2 acc[16][1];
 
         if constexpr (PROG == FZ_SKM12) {
             cp_wait<0>();
@@ -279,13 +272,13 @@ __global__ void __maxnreg__(REGS) fz_tplane_kernel(const __grid_constant__ FzTil
             }
             // s = S_1 S_2 a -> X
             w2.each([&](int kb, int u) {
-                line_item<K_SYN, RS, LP>(X, kb, nb2, u, p.td[0], acc);
-                store_trans<RS, LP>(Y, kb, u, acc);
+                line_item<K_SYN, RS, 2>(X, kb, nb2, u, p.td[0], acc);
+                store_trans<RS>(Y, kb, u, acc);
             });
             __syncthreads();
             w1.each([&](int kb, int u) {
-                line_item<K_SYN, RS, LP>(Y, kb, nb1, u, p.td[0], acc);
-                store_trans<RS, LP>(X, kb, u, acc);
+                line_item<K_SYN, RS, 2>(Y, kb, nb1, u, p.td[0], acc);
+                store_trans<RS>(X, kb, u, acc);
             });
             __syncthreads();
             // eight rows of four columns, as in the general form: the same chains of Ekin
@@ -404,10 +397,10 @@ __global__ void __maxnreg__(REGS) fz_tplane_kernel(const __grid_constant__ FzTil
             cp_wait<0>();
             __syncthreads();
             w2.each([&](int kb, int u) {
-                line_item<K_MFT, RS, LP>(Y, kb, nb2, u, p.td[0], acc);
+                line_item<K_MFT, RS, 2>(Y, kb, nb2, u, p.td[0], acc);
                 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const unsigned o = (2 * kb + h) * 8 * PlaneBuf<RS>::ROW + line_off<LP>(u, 2 * kb + h);
+                    const unsigned o = (2 * kb + h) * 8 * PlaneBuf<RS>::ROW + line_off<2>(u, 2 * kb + h);
                     #pragma unroll
                     for (int k = 0; k < 8; ++k) {
                         const float2 v = half_word(((Z + o) ^ (k << 4)) + k * PlaneBuf<RS>::ROW);
@@ -431,8 +424,8 @@ __global__ void __maxnreg__(REGS) fz_tplane_kernel(const __grid_constant__ FzTil
             if (more) fetch_plane<RS>(X, nx.S->in2 + nx.base);
             cp_commit();
             w2.each([&](int kb, int u) {
-                line_item<K_ANA, RS, LP>(Y, kb, nb2, u, p.td[1], acc);
-                store_global<LP>(S.out + c.base, N1, kb, u, acc);
+                line_item<K_ANA, RS, 2>(Y, kb, nb2, u, p.td[1], acc);
+                store_global(S.out + c.base, N1, kb, u, acc);
             });
         }
         c = nx;
@@ -442,22 +435,23 @@ __global__ void __maxnreg__(REGS) fz_tplane_kernel(const __grid_constant__ FzTil
     }
 }
 
+size_t tplane_smem(FzShape s) { return (s.ctas > 0 ? 3 : 2) * (size_t)s.rs * s.rs * sizeof(float); }
+
 template <typename F>
 cudaError_t tplane_pick(int prog, FzShape s, F&& f) {
     if (prog == FZ_SKM12) switch (s.rs) {
-        case 128: return f(fz_tplane_kernel<FZ_SKM12, 128, 128, 2>);
-        case 96: return f(fz_tplane_kernel<FZ_SKM12, 96, 128, 2>);
-        case 64: return f(fz_tplane_kernel<FZ_SKM12, 64, 128, 2>);
-        case 32: return f(fz_tplane_kernel<FZ_SKM12, 32, 128, 2>);
+        case 128: return f(fz_tplane_kernel<FZ_SKM12, 128, 128>);
+        case 96: return f(fz_tplane_kernel<FZ_SKM12, 96, 128>);
+        case 64: return f(fz_tplane_kernel<FZ_SKM12, 64, 128>);
+        case 32: return f(fz_tplane_kernel<FZ_SKM12, 32, 128>);
         }
     if (prog == FZ_MFTA12) switch (s.rs) {
-        case 128: return f(fz_tplane_kernel<FZ_MFTA12, 128, 128, 2>);
-        case 96: return f(fz_tplane_kernel<FZ_MFTA12, 96, 96, 2>);
-        case 64: return f(fz_tplane_kernel<FZ_MFTA12, 64, 96, 2>);
+        case 128: return f(fz_tplane_kernel<FZ_MFTA12, 128, 128>);
+        case 96: return f(fz_tplane_kernel<FZ_MFTA12, 96, 96>);
+        case 64: return f(fz_tplane_kernel<FZ_MFTA12, 64, 96>);
         }
     return cudaErrorInvalidConfiguration;
 }
-size_t tplane_smem(FzShape s) { return (s.ctas > 0 ? 3 : 2) * (size_t)s.rs * s.rs * sizeof(float); }
 
 }  // namespace
 
@@ -477,9 +471,19 @@ FzShape fz_tplane_shape(int prog, int N1, int N2) {
 }
 
 cudaError_t prepare_tplane(int prog, FzShape s) {
-    return tplane_pick(prog, s, [&](auto* k) {
+    // large dynamic shared memory once per device and kernel
+    static std::atomic<unsigned long long> done[2][5];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = 1ull << (dev & 63);
+    std::atomic<unsigned long long>& d = done[prog == FZ_SKM12][s.rs / 32];
+    if (d.load() & bit) return cudaSuccess;
+    e = tplane_pick(prog, s, [&](auto* k) {
         return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tplane_smem(s));
     });
+    if (e == cudaSuccess) d.fetch_or(bit);
+    return e;
 }
 
 cudaError_t launch_tplane(int prog, const FzParams<float>& p, cudaStream_t st) {

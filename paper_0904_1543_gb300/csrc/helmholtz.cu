@@ -36,6 +36,7 @@
 #include <cuda_runtime.h>
 
 #include "dot_acc.cuh"
+#include "static_for.cuh"
 #include "wvl_internal.h"
 
 namespace wvl {
@@ -72,15 +73,6 @@ struct HzParams {
     int nblk;               // hz_step, hz_init: blocks per orbital
 };
 
-template <typename F, int... I>
-__device__ __forceinline__ void hz_for_impl(F&& f, std::integer_sequence<int, I...>) {
-    (f(std::integral_constant<int, I>{}), ...);
-}
-template <int N, typename F>
-__device__ __forceinline__ void hz_for(F&& f) {
-    hz_for_impl(f, std::make_integer_sequence<int, N>{});
-}
-
 // rowoff[HZ_PAD + j] = (j mod n) * stride for j in [-HZ_PAD, nr + HZ_PAD), nr = n rounded
 // up to whole items
 __device__ __forceinline__ void hz_rowoff(int* rowoff, int n, int stride) {
@@ -96,11 +88,11 @@ __device__ __forceinline__ void hz_rowoff(int* rowoff, int n, int stride) {
 __device__ __forceinline__ void hz_col_sum(const float* __restrict__ base, const int* __restrict__ ro,
                                            const float (&f)[2][48], float2 (&acc)[HZ_RC][2]) {
     // window row j is row r0 - HZ_LO + j; rows k and k + 1 (k even) both take j = k .. k + 45
-    hz_for<HZ_RC - 2 + HZ_NT>([&](auto jc) {
+    static_for<HZ_RC - 2 + HZ_NT>([&](auto jc) {
         constexpr int j = decltype(jc)::value;
         const float4 v = *reinterpret_cast<const float4*>(base + ro[j]);
         const float2 a = make_float2(v.x, v.y), b = make_float2(v.z, v.w);
-        hz_for<HZ_RC>([&](auto kc) {
+        static_for<HZ_RC>([&](auto kc) {
             constexpr int k = decltype(kc)::value;
             constexpr int t = j - (k & ~1);
             if constexpr (t >= 0 && t < HZ_NT) {
@@ -261,15 +253,15 @@ __global__ void __maxnreg__(80) hz_plane_kernel(const __grid_constant__ HzParams
             off[i] = 4 * c;
             if (++c == ncv) c = 0;
         }
-        hz_for<HZ_RC>([&](auto kc) {
+        static_for<HZ_RC>([&](auto kc) {
             constexpr int k = decltype(kc)::value;
             const float* const row = X + rowoff[HZ_PAD + r0 + k];
-            hz_for<13>([&](auto ic) {
+            static_for<13>([&](auto ic) {
                 constexpr int i = decltype(ic)::value;
                 const float4 v = *reinterpret_cast<const float4*>(row + off[i]);
                 const float e[4] = {v.x, v.y, v.z, v.w};
                 // outputs 2m, 2m + 1 take input j with the pair j - 2m - 2
-                hz_for<8>([&](auto jm) {
+                static_for<8>([&](auto jm) {
                     constexpr int j = 4 * i + decltype(jm)::value / 2, m = decltype(jm)::value % 2;
                     constexpr int t = j - 2 * m - 2;
                     if constexpr (t >= 0 && t < HZ_NT)

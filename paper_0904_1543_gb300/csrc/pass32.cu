@@ -32,11 +32,11 @@
 #include <algorithm>
 #include <atomic>
 #include <type_traits>
-#include <utility>
 
 #include <cuda_runtime.h>
 
 #include "pass_kernel.cuh"
+#include "static_for.cuh"
 
 namespace wvl {
 namespace {
@@ -49,15 +49,6 @@ constexpr int P32_SMEM = 200 * 1024;
 // CTAs have 32 to 128 threads (64 orbitals with density on a free 16^3 box, in the same
 // groups: 172 us at 80, 116 at 128; on a periodic 37x45x51 cell 364 and 274)
 __host__ __device__ constexpr int p32_ctas(int mode) { return mode == M_POT ? 2 : 3; }
-
-template <typename F, int... I>
-__device__ __forceinline__ void p32_for_impl(F&& f, std::integer_sequence<int, I...>) {
-    (f(std::integral_constant<int, I>{}), ...);
-}
-template <int N, typename F>
-__device__ __forceinline__ void p32_for(F&& f) {
-    p32_for_impl(f, std::make_integer_sequence<int, N>{});
-}
 
 __host__ __device__ constexpr int p32_ltp(int LT) { return LT + 4; }   // row stride, 16-byte rows
 // rows of the tile: the windows of ceil(n / 8) chunks
@@ -334,11 +325,11 @@ __global__ void __launch_bounds__(P32_THREADS, p32_ctas(MODE)) pass32_kernel(con
                 const float* const win = X + i0 * LTP + l0;
                 #pragma unroll
                 for (int r = 0; r < R; ++r) acc[r][0] = acc[r][1] = make_float2(0.f, 0.f);
-                p32_for<W>([&](auto jc) {
+                static_for<W>([&](auto jc) {
                     constexpr int j = decltype(jc)::value;
                     const float4 q = *reinterpret_cast<const float4*>(win + j * LTP);
                     const float2 q0 = make_float2(q.x, q.y), q1 = make_float2(q.z, q.w);
-                    p32_for<R>([&](auto rc) {
+                    static_for<R>([&](auto rc) {
                         constexpr int r = decltype(rc)::value;
                         constexpr int k = j - r - ((r & 1) ? KT<KIND>::OFF1 : KT<KIND>::OFF0);
                         if constexpr (tap_on<KIND>(k)) {

@@ -208,8 +208,9 @@ inline int fz_plane_rs(int N1) {
 //   one CTA       512 threads, 128 registers: 128^2 812 / 432 (256 threads 825 / 463), 120^2
 //                 770 / 413 (840 / 465)
 //   two           256; 320 at 96 registers where that saves a second round of column items
-//                 (96^2, 288 items: 456 / 219 against 460 / 236); 112^2 706 / 355, where
-//                 320 takes 720 / 345
+//                 (88x112, 308 items: 538 / 266 against 554 / 273; 96x104 520 / 252
+//                 against 524 / 257; 128x72 394 / 201 against 386 / 203); 112^2 706 / 355,
+//                 where 320 takes 720 / 345
 //   three         160: 88^2 376 / 187 (256: 391 / 202)
 //   four and more 128, at 96 registers from five on: 80^2 279 / 136 (309 / 158), 64^2
 //                 267 / 123 (310 / 163); fewer where a plane has fewer items: 48^2 315 / 146
