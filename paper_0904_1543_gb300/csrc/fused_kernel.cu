@@ -280,9 +280,9 @@ __device__ __forceinline__ void col_item(const T* __restrict__ src, const int* _
 template <int PROG>
 __host__ __device__ constexpr int fz_cthreads() { return PROG == FZ_TA3 ? 2 * FZ_CTHREADS : FZ_CTHREADS; }
 
-template <typename T, int PROG, int REGS>
-__global__ void __maxnreg__(REGS)
-fz_plane_kernel(const __grid_constant__ FzParams<T> p) {
+// THREADS: threads of the CTA, for the plane's copy (0: at run time)
+template <typename T, int PROG, int THREADS>
+__device__ __forceinline__ void fz_plane(const FzParams<T>& p) {
     constexpr int VEC = 16 / (int)sizeof(T);
     constexpr int RC = FZ_RC;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -303,7 +303,7 @@ fz_plane_kernel(const __grid_constant__ FzParams<T> p) {
     const int ncv = N1 / VEC;
     const int nitems = (N2 / RC) * ncv;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int NWARP = (int)(blockDim.x >> 5);
+    const int NWARP = THREADS > 0 ? THREADS / 32 : (int)(blockDim.x >> 5);
 
     // the plane, row I2 -> X + I2 RS (a warp per row, lanes over its vectors)
     {
@@ -461,6 +461,18 @@ fz_plane_kernel(const __grid_constant__ FzParams<T> p) {
                 stv(S.out + pbase + (long long)(r0 + kk) * N1 + cv * VEC, acc[kk]);
         }
     }
+}
+
+template <typename T, int PROG, int REGS>
+__global__ void __maxnreg__(REGS) fz_plane_kernel(const __grid_constant__ FzParams<T> p) {
+    fz_plane<T, PROG, 0>(p);
+}
+// 256 threads, as launch bounds instead of a register cap: 979 us of SYN3 + SKM12 on 104^2
+// planes (144 orbitals), 995 as an instance of the kernel above, 1016 with every loop's step
+// folded to 256 too
+template <typename T, int PROG>
+__global__ void __launch_bounds__(256) fz_plane256_kernel(const __grid_constant__ FzParams<T> p) {
+    fz_plane<T, PROG, 256>(p);
 }
 
 // ----------------------------------------------------------- column kernels
@@ -827,6 +839,13 @@ constexpr bool fz_is_plane() { return PROG == FZ_SKM12 || PROG == FZ_MFTA12; }
 
 constexpr int FZ_SMEM_OPTIN = 224 * 1024;   // under the opt-in limit with the static reduction buffer
 
+// the plane kernel of a register cap (0: of 256 threads)
+template <typename T, int PROG, int REGS>
+auto fz_plane_ptr() {
+    if constexpr (REGS == 0) return &fz_plane256_kernel<T, PROG>;
+    else return &fz_plane_kernel<T, PROG, REGS>;
+}
+
 template <typename T, int PROG, int REGS>
 cudaError_t fz_ensure_attr() {
     static std::atomic<unsigned long long> done{0};
@@ -836,7 +855,7 @@ cudaError_t fz_ensure_attr() {
     const unsigned long long bit = 1ull << (dev & 63);
     if (!(done.load() & bit)) {
         if constexpr (fz_is_plane<PROG>())
-            err = cudaFuncSetAttribute(fz_plane_kernel<T, PROG, REGS>,
+            err = cudaFuncSetAttribute(fz_plane_ptr<T, PROG, REGS>(),
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, FZ_SMEM_OPTIN);
         else
             err = cudaFuncSetAttribute(fz_col_kernel<T, PROG>,
@@ -851,7 +870,7 @@ template <typename T, int PROG, int REGS>
 cudaError_t fz_plane_launch(const FzParams<T>& p, int threads, size_t smem, cudaStream_t st) {
     cudaError_t err = fz_ensure_attr<T, PROG, REGS>();
     if (err != cudaSuccess) return err;
-    fz_plane_kernel<T, PROG, REGS><<<dim3((unsigned)p.njobs), dim3(threads), smem, st>>>(p);
+    fz_plane_ptr<T, PROG, REGS>()<<<dim3((unsigned)p.njobs), dim3(threads), smem, st>>>(p);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -875,10 +894,11 @@ cudaError_t fz_launch(const FzParams<T>& p, size_t smem, cudaStream_t st) {
                 tap_pairs<K_MFT>(q.tap[0], q.tp[0]);
                 tap_pairs<K_ANA>(q.tap[1], q.tp[1]);
             }
+            if (s.threads == 256) return fz_plane_launch<T, PROG, 0>(q, 256, smem, st);
             if (s.regs == 96) return fz_plane_launch<T, PROG, 96>(q, s.threads, smem, st);
             return fz_plane_launch<T, PROG, 128>(q, s.threads, smem, st);
         } else {
-            return fz_plane_launch<T, PROG, 255>(p, s.threads, smem, st);
+            return fz_plane_launch<T, PROG, 0>(p, 256, smem, st);
         }
     } else {
         cudaError_t err = fz_ensure_attr<T, PROG, 0>();
@@ -923,9 +943,10 @@ cudaError_t prepare_fused_kernels() {
     if ((e = fz_ensure_attr<T, FZ_SYN3, 0>()) != cudaSuccess) return e;
     if ((e = fz_ensure_attr<T, FZ_POT3, 0>()) != cudaSuccess) return e;
     if ((e = fz_ensure_attr<T, FZ_TA3, 0>()) != cudaSuccess) return e;
+    if ((e = fz_ensure_attr<T, FZ_SKM12, 0>()) != cudaSuccess) return e;
+    if ((e = fz_ensure_attr<T, FZ_MFTA12, 0>()) != cudaSuccess) return e;
     if constexpr (sizeof(T) == 8) {
-        if ((e = fz_ensure_attr<T, FZ_SKM12, 255>()) != cudaSuccess) return e;
-        return fz_ensure_attr<T, FZ_MFTA12, 255>();
+        return cudaSuccess;
     } else {
         if ((e = fz_ensure_attr<T, FZ_SKM12, 96>()) != cudaSuccess) return e;
         if ((e = fz_ensure_attr<T, FZ_SKM12, 128>()) != cudaSuccess) return e;

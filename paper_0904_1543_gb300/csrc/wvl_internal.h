@@ -218,10 +218,11 @@ inline int fz_plane_rs(int N1) {
 // More planes per SM overlap one's loads and barriers with another's filters.  A CTA's
 // warps are a multiple of four where CTAs share an SM's registers closely (288 threads
 // at 112 registers leave one CTA per SM: 579 / 338).  Launches of at most two CTAs per SM keep
-// 256 threads: there a plane's own time counts.  FP64 planes are bound by the FP64 pipe.
+// 256 threads: there a plane's own time counts.  FP64 planes are bound by the FP64 pipe.  (256
+// threads have a kernel of their own.)
 template <typename T>
 inline FzShape fz_plane_shape(int prog, int N1, int N2, long long planes) {
-    if (sizeof(T) == 8) return {256, 255};
+    if (sizeof(T) == 8) return {256, 128};
     if (planes <= 2 * 152) return {256, 128};
     const FzShape ts = fz_tplane_shape(prog, N1, N2);
     if (ts.rs > 0) return ts;
