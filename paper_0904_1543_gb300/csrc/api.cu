@@ -196,7 +196,10 @@ static int rowlen_of(int n, int R, const KindGeom& g, size_t elt) {
 // box (45^3 points), 2 orbitals 9.4, 11.1 / 6.5, 7.9; 4 orbitals 11.2, 13.0 / 7.6, 8.1; 8
 // orbitals 17.8, 16.3 / 10.9, 9.0; free 32^3, 8 orbitals 108, 52 / 56, 32; 64 orbitals
 // 453, 283 / 391, 211.  With a density lines of fewer than 32 outputs stay row-wise: a tile
-// has no full warp then (24 outputs, 64 orbitals: 31 against 36).
+// has no full warp then (24 outputs, 64 orbitals: 31 against 36).  The compressed passes of
+// less than 5e5 points are row-wise for the same reason: synthesis pass 1 and analysis pass 3
+// on 20x21x31, 2 orbitals 4.3, 6.0 and 5.3, 7.6; 8 orbitals 8.2, 7.0 and 10.2, 8.2; on 37x45x51,
+// 2 orbitals 9.6, 7.9 and 13.8, 8.5.
 template <typename T>
 static bool use_pass32(const PassCall<T>& c) {
     if (sizeof(T) != 4) return false;
@@ -214,9 +217,12 @@ static bool use_pass32(const PassCall<T>& c) {
         return points >= (plain ? 100000 : 500000) && 2 * longer >= points;
     }
     if (c.mode != M_UNCOMP && c.mode != M_COMP) return false;
-    for (const auto& d : c.segs)
+    long long points = 0;
+    for (const auto& d : c.segs) {
         if (d.s.mapc != nullptr || d.s.bx1 != 0 || d.gn != 0) return false;
-    return true;
+        points += d.s.P * d.s.norb;
+    }
+    return points >= 500000;
 }
 
 // Orbitals per group of an FP32 potential pass of pass32.cu with a density, at most gmax
