@@ -1,6 +1,7 @@
 // Dispatch of the pass kernels for one element type (included once per type
 // by kernels_f64.cu / kernels_f32.cu so the two compile in parallel).
 #pragma once
+#include <algorithm>
 #include <atomic>
 
 #include "pass_kernel.cuh"
@@ -24,24 +25,27 @@ static cudaError_t ensure_attr() {
     return cudaSuccess;
 }
 
-// Persistent launch: as many CTAs as fit on the device at once (never more
-// than there are work units); each walks its units with a stride of the grid.
+// One CTA per work unit, or persistent: as many CTAs as fit on the device at once (never
+// more than there are work units), each walking its units with a stride of the grid.
+// (Only that asks for the occupancy: a microsecond or so of every launch.)
 template <typename T, int KIND, int MODE, int R>
 static cudaError_t launch_one(const PassParams<T>& p, long long nunits, size_t smem,
                               cudaStream_t st, bool persistent) {
     cudaError_t err = ensure_attr<T, KIND, MODE, R>();
     if (err != cudaSuccess) return err;
     if (nunits <= 0) return cudaSuccess;
-    int dev = 0, nsm = 0, occ = 0;
-    if ((err = cudaGetDevice(&dev)) != cudaSuccess) return err;
-    if ((err = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-        return err;
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, pass_kernel<T, KIND, MODE, R>,
-                                                        NTHREADS, smem);
-    if (err != cudaSuccess) return err;
-    if (occ < 1) return cudaErrorInvalidConfiguration;
-    long long grid = persistent ? (long long)occ * nsm : nunits;
-    if (grid > nunits) grid = nunits;
+    long long grid = nunits;
+    if (persistent) {
+        int dev = 0, nsm = 0, occ = 0;
+        if ((err = cudaGetDevice(&dev)) != cudaSuccess) return err;
+        if ((err = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+            return err;
+        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, pass_kernel<T, KIND, MODE, R>,
+                                                            NTHREADS, smem);
+        if (err != cudaSuccess) return err;
+        if (occ < 1) return cudaErrorInvalidConfiguration;
+        grid = std::min(nunits, (long long)occ * nsm);
+    }
     if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     if constexpr (sizeof(T) == 4) {
         PassParams<T> q = p;
