@@ -29,9 +29,9 @@
  *   FP32 chain of at most 32 products of convolution outputs, converted
  *   exactly (the fused potential kernel first sums a warp's 32 chains in a
  *   compensated single pair, ~48-bit); scalar products (wvl_overlap,
- *   wvl_dot) form every product and sum in double; rho over orbitals is
- *   carried per thread in compensated single (~48-bit) and in double from
- *   there on.
+ *   wvl_dot, the preconditioner's) are accurate to double, each in its own
+ *   way (see there); rho over orbitals is carried per thread in compensated
+ *   single (~48-bit) and in double from there on.
  *   WVL_F64_EMU -- arrays as WVL_F64; every 1D convolution sum of the
  *   passes (Eqs. 1dconvtrans, kinetic1d) is evaluated on the FP16 tensor
  *   cores instead of the FP64 pipe: operands split into six signed 10-bit

@@ -368,8 +368,8 @@ def _overlap_ws(prec, na, nb, ln, device):
 
 def overlap(a, b=None):
     """Scalar products <a_i|b_j> of compressed orbitals (rows of a and b; b
-    defaults to a) as a float64 (na, nb) device tensor: FP64 products and
-    accumulation whatever the coefficients' precision."""
+    defaults to a) as a float64 (na, nb) device tensor, accurate to an FP64 sum of
+    FP64 products whatever the coefficients' precision."""
     b = a if b is None else b
     if a.dtype != b.dtype:
         raise TypeError("a and b must have the same dtype")
@@ -388,7 +388,7 @@ def overlap(a, b=None):
 
 
 def dot(a, b):
-    """Per-orbital scalar products <a_o|b_o> (float64, FP64 accumulation)."""
+    """Per-orbital scalar products <a_o|b_o> (float64, accurate to FP64 sums)."""
     if a.shape != b.shape or a.dtype != b.dtype:
         raise ValueError("a and b must have the same shape and dtype")
     a2 = a.reshape(a.shape[0], -1)

@@ -526,7 +526,7 @@ enum Chain { CHAIN_AUTO = 0, CHAIN_PASSES = 1, CHAIN_FUSED = 2 };
 static size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 // partial sums per orbital of the passes that write them (the last axis):
-// tiles of LT_MIN lines, or 128-line tiles x 32-output windows when emulated
+// tiles of LT_MIN lines, or 128-line tiles x 16-output windows when emulated
 static long long tiles_max(const int Nf[3]) {
     long long N = (long long)Nf[1] * Nf[0];
     const long long emu_tiles = (N + emu::M - 1) / emu::M * ((Nf[2] + emu::NWIN - 1) / emu::NWIN);

@@ -132,14 +132,14 @@ __device__ __forceinline__ bool next_job(const PassParams<double>& p, int mode, 
 
 // The 26 digit pairs of the canonical schedule (diagonal d = 2..8, i.e.
 // dq + fp = d - 2 <= 6, accumulating in tensor-memory columns (d - 2) N..)
-// as 6 data digits x 3 K-steps: the MMA of data digit dq multiplies it by the
+// as 6 data digits x 2 K-steps (3 for the kinetic filter): the MMA of data digit dq multiplies it by the
 // filter digits fp = 0 .. 6 - dq side by side (N (7 - dq) columns from column
 // dq N), so one instruction adds the products of every pair with that dq to
 // their diagonals.  The first one (dq = 0, K-step 0) also meets the zero
 // block (fp = 6) and so starts all seven accumulators.  Every exact
 // diagonal's partial sums stay integers below 2^24 in any order, so the
 // order of the pairs does not change the result.  K-step k reads the data
-// planes' slab slot (slot0 + k) mod 3; the shared-memory descriptors are base
+// planes' slab slot (slot0 + k) mod the number of K-steps; the shared-memory descriptors are base
 // + compile-time offsets.
 template <int KIND, int MODE>
 __device__ __forceinline__ void issue_window_mmas(uint32_t tm, uint32_t a_base, uint32_t b_base,
