@@ -28,14 +28,14 @@
 // note that exponent per line of the next pass as they store (warp_tops, emu.cuh: hand_slots).
 // Where an FP64 array comes in, a line's exponent is the largest of a first read.
 // One scale for all lines that cross the same source lines would do without the notes and
-// the shifts to the left (23.6 ms instead of 25.0 per headline step), but lines
+// the shifts to the left (23.6 ms instead of 24.9 per headline step), but lines
 // far below their neighbours then lose their bits (a Gaussian of 2.5 points, modelled: at 1e-6
 // of its peak off two axes, 2e-12 of the element instead of 6e-15).  H psi of random coefficients:
 // 1.2e-16 in the 2-norm (FP64 kernels 4.2e-16).
 // Per headline step (192 orbitals): 30.9 ms with windows of 32 outputs, two CTAs per SM;
 // 29.2 with 16 outputs and three; 28.5 with fields masked and completed in one
 // operation; 24.7 with the integers and the copies, 23.6 with the kinetic passes' rows,
-// 25.0 with a scale per line (integers and copies: neither alone gains,
+// 24.9 with a scale per line (integers and copies: neither alone gains,
 // without the scan's first read the slabs' loads wait for HBM, and copies of FP64 arrays leave
 // the scan; an L2 prefetch of the next slab gave 27.5, of the next tile 29.4, a
 // register prefetch of the next slab 31.7).
@@ -226,12 +226,6 @@ struct HandOut {
     int* top0;   // the same entry in slot 0, which the others take
     int step, more;
 };
-// position of the highest bit that differs from the sign; -1 for 0 and -1
-__device__ __forceinline__ int top_bit(int x) {
-    int p;
-    asm("bfind.s32 %0, %1;" : "=r"(p) : "r"(x));
-    return p;
-}
 // exponents as pairs of 16 bits, one pair per two outputs
 __device__ __forceinline__ unsigned pair16(int a, int b) { return __byte_perm((unsigned)a, (unsigned)b, 0x5410); }
 constexpr int HAND_NONE = -30000;
@@ -306,7 +300,7 @@ __device__ __forceinline__ double window_epilogue(const Seg<double>& Sg, uint32_
         co = cc0 + Sg.ncoarse + 7LL * cx + mu12 + 3 + i2 * so_;
     }
     if (OUTI ? lt <= (er & ~31) : !row_ok) return 0.0;   // (integer output: whole warps)
-    unsigned pe[NH / 2], nz = 0;   // exponents of the integer outputs; any of them not zero
+    unsigned pe[NH / 2];   // exponents of the integer outputs
     {
 #pragma unroll
         for (int c = 0; c < NH; ++c) {
@@ -331,9 +325,8 @@ __device__ __forceinline__ double window_epilogue(const Seg<double>& Sg, uint32_
             const long long oi = oi0 + (long long)c * NL;
             if constexpr (OUTI) {
                 // the next pass reads the integer, the line's scale and the largest exponent
-                // of its own lines
-                const int e = gl + 33 + top_bit((int)(t >> 32));
-                nz |= (unsigned)t | (unsigned)(t >> 32);
+                // of its own lines, |t| 2^gl <= 2^e (0: 2^-126 of the scale)
+                const int e = gl + hand_bits(__ll2float_rn(t));
                 pe[c / 2] = c & 1 ? pair16((int)pe[c / 2], e) : (unsigned)e;
                 if (row_ok) reinterpret_cast<long long*>(Sg.out)[oi] = t;
                 continue;
@@ -387,24 +380,9 @@ __device__ __forceinline__ double window_epilogue(const Seg<double>& Sg, uint32_
         }
     }
     if constexpr (OUTI) {
-        if (!row_ok || nz == 0)
+        if (!row_ok)
 #pragma unroll
             for (int k = 0; k < NH / 2; ++k) pe[k] = pair16(HAND_NONE, HAND_NONE);
-        // integers without a high word (zeros among them): the exact exponents
-        const unsigned small = __vmins2(__vmins2(pe[0], pe[1]), __vmins2(pe[2], pe[3]));
-        if (__any_sync(0xffffffffu, row_ok && nz != 0 && min((int)(short)small, (int)small >> 16) <= gl + 32)) {
-            int e[NH];
-#pragma unroll
-            for (int c = 0; c < NH; ++c) {
-                e[c] = HAND_NONE;
-                if (row_ok && o0 + c < n) {
-                    const long long t = reinterpret_cast<const long long*>(Sg.out)[oi0 + (long long)c * NL];
-                    if (t != 0) e[c] = gl + 64 - __clzll(t ^ (t >> 63));
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < NH / 2; ++k) pe[k] = pair16(e[2 * k], e[2 * k + 1]);
-        }
         const HandOut ho = hos[er >> 5];
         auto tops = [&](const unsigned (&m)[NH / 2], int* top) {
             warp_tops(m, [&](int c, int e) {

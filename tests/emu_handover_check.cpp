@@ -2,6 +2,7 @@
 // (emu.cuh), compiled and run by tests/test_emu_handover.py on the CPU:
 //  - requantize() where the line's largest value lies below the scale of an integer, so that
 //    the shift goes to the left, is exact: X = t 2^(g + QBITS - E);
+//  - hand_bits() bounds an integer's magnitude, by less than a factor of four;
 //  - every line of n elements is covered by hand_slots(n) warps of 32 source lines at most,
 //    each writing one slot of its own, and the slots, scales and line exponents of an
 //    operator's passes fit into one FP64 array of the cell, for any extents.
@@ -36,6 +37,16 @@ int main() {
     for (int E = -960; E < 1000; E += 7)   // zeros of lines of any other scale
         for (int g = -1100; g < 1000; g += 13)
             if (requantize(0, g, E) != DBIAS && fails++ < 10) std::printf("FAIL zero g %d E %d\n", g, E);
+    for (int it = 0; it < 2000000; ++it) {   // the exponent of an integer, a tight upper bound
+        const int bits = 1 + (int)(rng() % 60);
+        long long t = (long long)(rng() >> (64 - bits));
+        if (it % 3 == 0) t = (1LL << bits) - (it % 2);
+        if (t == 0) continue;
+        const int b = hand_bits((float)(rng() & 1 ? -t : t));
+        if ((__int128)t > (__int128)1 << b || (__int128)4 * t <= (__int128)1 << b)
+            if (fails++ < 10) std::printf("FAIL bits t %lld b %d\n", t, b);
+    }
+    if (hand_bits(0.f) != -126) ++fails;
     for (int n = 2; n <= 1024; n += 2) {
         // lines c of n source lines each: the warps that share one, and their slots
         for (int c = 0; c < 40; ++c) {
