@@ -463,13 +463,18 @@ __device__ __forceinline__ void fz_plane(const FzParams<T>& p) {
     }
 }
 
+// registers capped at REGS; as the compiler allocates them (REGS = 0, at most 512 threads): MFTA12
+// takes 65 and 122 under a cap of 128, at which it is 13 % slower
 template <typename T, int PROG, int REGS>
 __global__ void __maxnreg__(REGS) fz_plane_kernel(const __grid_constant__ FzParams<T> p) {
     fz_plane<T, PROG, 0>(p);
 }
-// 256 threads, as launch bounds instead of a register cap: 979 us of SYN3 + SKM12 on 104^2
-// planes (144 orbitals), 995 as an instance of the kernel above, 1016 with every loop's step
-// folded to 256 too
+template <typename T, int PROG>
+__global__ void __launch_bounds__(512) fz_plane512_kernel(const __grid_constant__ FzParams<T> p) {
+    fz_plane<T, PROG, 0>(p);
+}
+// 256 threads: 979 us of SYN3 + SKM12 on 104^2 planes (144 orbitals), 995 with a cap of 128
+// registers, 1016 with every loop's step folded to 256 too
 template <typename T, int PROG>
 __global__ void __launch_bounds__(256) fz_plane256_kernel(const __grid_constant__ FzParams<T> p) {
     fz_plane<T, PROG, 256>(p);
@@ -839,14 +844,15 @@ constexpr bool fz_is_plane() { return PROG == FZ_SKM12 || PROG == FZ_MFTA12; }
 
 constexpr int FZ_SMEM_OPTIN = 224 * 1024;   // under the opt-in limit with the static reduction buffer
 
-// the plane kernel of a register cap (0: of 256 threads)
-template <typename T, int PROG, int REGS>
+// the plane kernel of 256 threads (K = 256), of any number as compiled (0), of a register cap
+template <typename T, int PROG, int K>
 auto fz_plane_ptr() {
-    if constexpr (REGS == 0) return &fz_plane256_kernel<T, PROG>;
-    else return &fz_plane_kernel<T, PROG, REGS>;
+    if constexpr (K == 256) return &fz_plane256_kernel<T, PROG>;
+    else if constexpr (K == 0) return &fz_plane512_kernel<T, PROG>;
+    else return &fz_plane_kernel<T, PROG, K>;
 }
 
-template <typename T, int PROG, int REGS>
+template <typename T, int PROG, int K>
 cudaError_t fz_ensure_attr() {
     static std::atomic<unsigned long long> done{0};
     int dev = 0;
@@ -855,7 +861,7 @@ cudaError_t fz_ensure_attr() {
     const unsigned long long bit = 1ull << (dev & 63);
     if (!(done.load() & bit)) {
         if constexpr (fz_is_plane<PROG>())
-            err = cudaFuncSetAttribute(fz_plane_ptr<T, PROG, REGS>(),
+            err = cudaFuncSetAttribute(fz_plane_ptr<T, PROG, K>(),
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, FZ_SMEM_OPTIN);
         else
             err = cudaFuncSetAttribute(fz_col_kernel<T, PROG>,
@@ -866,11 +872,11 @@ cudaError_t fz_ensure_attr() {
     return cudaSuccess;
 }
 
-template <typename T, int PROG, int REGS>
+template <typename T, int PROG, int K>
 cudaError_t fz_plane_launch(const FzParams<T>& p, int threads, size_t smem, cudaStream_t st) {
-    cudaError_t err = fz_ensure_attr<T, PROG, REGS>();
+    cudaError_t err = fz_ensure_attr<T, PROG, K>();
     if (err != cudaSuccess) return err;
-    fz_plane_ptr<T, PROG, REGS>()<<<dim3((unsigned)p.njobs), dim3(threads), smem, st>>>(p);
+    fz_plane_ptr<T, PROG, K>()<<<dim3((unsigned)p.njobs), dim3(threads), smem, st>>>(p);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -894,11 +900,12 @@ cudaError_t fz_launch(const FzParams<T>& p, size_t smem, cudaStream_t st) {
                 tap_pairs<K_MFT>(q.tap[0], q.tp[0]);
                 tap_pairs<K_ANA>(q.tap[1], q.tp[1]);
             }
-            if (s.threads == 256) return fz_plane_launch<T, PROG, 0>(q, 256, smem, st);
-            if (s.regs == 96) return fz_plane_launch<T, PROG, 96>(q, s.threads, smem, st);
-            return fz_plane_launch<T, PROG, 128>(q, s.threads, smem, st);
+            if (s.threads == 256) return fz_plane_launch<T, PROG, 256>(q, 256, smem, st);
+            if constexpr (PROG == FZ_SKM12)
+                if (s.regs == 96) return fz_plane_launch<T, PROG, 96>(q, s.threads, smem, st);
+            return fz_plane_launch<T, PROG, 0>(q, s.threads, smem, st);
         } else {
-            return fz_plane_launch<T, PROG, 0>(p, 256, smem, st);
+            return fz_plane_launch<T, PROG, 256>(p, 256, smem, st);
         }
     } else {
         cudaError_t err = fz_ensure_attr<T, PROG, 0>();
@@ -943,15 +950,14 @@ cudaError_t prepare_fused_kernels() {
     if ((e = fz_ensure_attr<T, FZ_SYN3, 0>()) != cudaSuccess) return e;
     if ((e = fz_ensure_attr<T, FZ_POT3, 0>()) != cudaSuccess) return e;
     if ((e = fz_ensure_attr<T, FZ_TA3, 0>()) != cudaSuccess) return e;
-    if ((e = fz_ensure_attr<T, FZ_SKM12, 0>()) != cudaSuccess) return e;
-    if ((e = fz_ensure_attr<T, FZ_MFTA12, 0>()) != cudaSuccess) return e;
+    if ((e = fz_ensure_attr<T, FZ_SKM12, 256>()) != cudaSuccess) return e;
+    if ((e = fz_ensure_attr<T, FZ_MFTA12, 256>()) != cudaSuccess) return e;
     if constexpr (sizeof(T) == 8) {
         return cudaSuccess;
     } else {
         if ((e = fz_ensure_attr<T, FZ_SKM12, 96>()) != cudaSuccess) return e;
-        if ((e = fz_ensure_attr<T, FZ_SKM12, 128>()) != cudaSuccess) return e;
-        if ((e = fz_ensure_attr<T, FZ_MFTA12, 96>()) != cudaSuccess) return e;
-        if ((e = fz_ensure_attr<T, FZ_MFTA12, 128>()) != cudaSuccess) return e;
+        if ((e = fz_ensure_attr<T, FZ_SKM12, 0>()) != cudaSuccess) return e;
+        if ((e = fz_ensure_attr<T, FZ_MFTA12, 0>()) != cudaSuccess) return e;
         for (int rs = 32; rs <= 128; rs += 32)
             for (int prog : {FZ_SKM12, FZ_MFTA12}) {
                 const FzShape s = fz_tplane_shape(prog, rs, rs);

@@ -201,39 +201,52 @@ inline int fz_plane_rs(int N1) {
     return w * v;
 }
 // Square FP32 planes of 32 to 128 points a side in steps of 32 take the transposing form
-// (fused_plane.cu, with both sides measured).  The others: threads and register cap of a
-// plane kernel, by the CTAs whose two planes fit in an
-// SM's shared memory.  FP32, microseconds of SYN3 + SKM12 / MFTA12 per call of 64 orbitals
-// (48 at 128^2, 128 at 64^2, 256 at 48^2, 512 at 32^2):
-//   one CTA       512 threads, 128 registers: 128^2 812 / 432 (256 threads 825 / 463), 120^2
-//                 770 / 413 (840 / 465)
-//   two           256; 320 at 96 registers where that saves a second round of column items
-//                 (88x112, 308 items: 538 / 266 against 554 / 273; 96x104 520 / 252
-//                 against 524 / 257; 128x72 394 / 201 against 386 / 203); 112^2 706 / 355,
-//                 where 320 takes 720 / 345
-//   three         160: 88^2 376 / 187 (256: 391 / 202)
-//   four and more 128, at 96 registers from five on: 80^2 279 / 136 (309 / 158), 64^2
-//                 267 / 123 (310 / 163); fewer where a plane has fewer items: 48^2 315 / 146
-//                 (403 / 230), 32^2 150 / 78 (345 / 225)
-// More planes per SM overlap one's loads and barriers with another's filters.  A CTA's
-// warps are a multiple of four where CTAs share an SM's registers closely (288 threads
-// at 112 registers leave one CTA per SM: 579 / 338).  Launches of at most two CTAs per SM keep
-// 256 threads: there a plane's own time counts.  FP64 planes are bound by the FP64 pipe.  (256
-// threads have a kernel of their own.)
+// (fused_plane.cu, with both sides measured).  The others: threads of a plane kernel, by the
+// CTAs whose two planes fit in an SM's shared memory and by the column items of a plane (8 rows
+// of a 16-byte column; a last round of few items wastes the CTA); registers as compiled, or
+// capped at 96 where that lets one more CTA in.  More planes per SM overlap one's loads and
+// barriers with another's filters.  FP32, microseconds per call of 2560 planes of 40 (of 640, one
+// figure each, for SYN3 + SKM12 / MFTA12), with 256 threads and as chosen:
+//   one CTA       512: 120^2 404 / 212 and 378 / 186
+//   two, three    256 (80x88, 220 items: 177 / 75, with 160 185 / 84).  SKM12 160 where three
+//                 CTAs fit (256 threads leave registers for two), 256 would leave a second
+//                 round of at most 64 items, and rows are chunks of 8 (N1 no multiple of
+//                 16: twice the row items, which hide the fewer threads): 104x88, 286 items,
+//                 237 and 228; 88x96 218 and 203; 120x72 231 and 221; but 112x80 228 and 232,
+//                 88x112 (two CTAs) 255 and 289, and 480 planes of 104x88, two waves either
+//                 way, 64 and 72
+//   four          SKM12 128: 80^2 170 and 160; MFTA12 256
+//   five to seven 128 at 96 registers / 160: 72^2 174 / 67 and 154 / 63, 64x80 145 / 62 and
+//                 130 / 56
+//   eight, nine   128 at 96 / 128: 72x40 118 / 47 and 100 / 39, 56^2 113 / 46 and 99 / 40
+//   more          MFTA12 96: 48^2 43 and 33, 40^2 39 and 29; SKM12 at 96 registers 96 for 65 to
+//                 83 items, 48^2 92 and 77; 64 for fewer, 40^2 100 and 74 (96: 79); one
+//                 warp for planes of one warp's items
+// Launches of at most two planes per SM keep 256 threads, SKM12 at four CTAs and MFTA12 of at most
+// three (six for planes of one warp's items): there a plane's own time counts (320 planes of
+// 72^2: MFTA12 16.5 with 256, 18.5 with 160; of 32^2 9.7 and 12.3).  FP64
+// planes are bound by the FP64 pipe.  regs: 0 as compiled, else the cap.
 template <typename T>
 inline FzShape fz_plane_shape(int prog, int N1, int N2, long long planes) {
-    if (sizeof(T) == 8) return {256, 128};
-    if (planes <= 2 * 152) return {256, 128};
+    if (sizeof(T) == 8 || planes <= 2 * 152) return {256, 0};
     const FzShape ts = fz_tplane_shape(prog, N1, N2);
     if (ts.rs > 0) return ts;
-    const int smem = 2 * N2 * fz_plane_rs<T>(N1) * (int)sizeof(T) + 2048;
-    const int ctas = 227 * 1024 / smem;
+    // (static and reserved shared memory: 1792 bytes of the SM's 228 KB per CTA)
+    const int smem = 2 * N2 * fz_plane_rs<T>(N1) * (int)sizeof(T) + 1792;
+    const int ctas = 228 * 1024 / smem;
     const int items = (N2 / FZ_RC) * (N1 * (int)sizeof(T) / 16);
-    if (ctas <= 1) return {512, 128};
-    if (ctas == 2) return items > 256 && items <= 320 ? FzShape{320, 96} : FzShape{256, 128};
-    if (ctas == 3) return {160, 128};
-    if (ctas == 4) return {128, 128};
-    return {items <= 32 ? 32 : items <= 112 ? 64 : 128, 96};
+    if (ctas <= 1) return {512, 0};
+    if (prog == FZ_MFTA12) {
+        if (ctas <= 4 || planes <= (items <= 32 ? 6 : 3) * 152) return {256, 0};
+        return {items <= 32 ? 32 : ctas <= 7 ? 160 : ctas <= 9 ? 128 : 96, 0};
+    }
+    if (ctas == 2) return {256, 0};
+    if (ctas == 3) {
+        const bool fewer = (planes + 455) / 456 < (planes + 303) / 304;   // waves of three and of two
+        return {fewer && items > 256 && items <= 320 && N1 % 16 != 0 ? 160 : 256, 0};
+    }
+    if (ctas == 4) return {planes <= 3 * 152 ? 256 : 128, 0};
+    return {items <= 32 ? 32 : items <= 64 ? 64 : items < 84 ? 96 : 128, 96};
 }
 template <typename T>
 size_t fz_smem(int prog, int N1, int N2, int N3);

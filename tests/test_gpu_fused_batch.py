@@ -19,7 +19,11 @@ def W():
     return W
 
 
-@pytest.mark.parametrize("n", [(16, 16, 20), (32, 32, 16), (48, 48, 20), (64, 64, 16), (40, 40, 16), (24, 36, 16)])
+# transposing planes, then one of every thread count of the general kernels: 512, 256, 160
+# (SKM12), 128, 160 (MFTA12), 128, 96 and 64 threads
+@pytest.mark.parametrize("n", [(16, 16, 20), (32, 32, 16), (48, 48, 20), (64, 64, 16),
+                               (60, 60, 16), (44, 40, 16), (52, 44, 16), (40, 40, 16), (36, 32, 16), (24, 36, 16),
+                               (36, 20, 16), (24, 24, 20), (20, 16, 20), (16, 20, 16)])
 def test_same_bits(W, n):
     import torch
     g = W.Grid(n, (0.25, 0.3, 0.2))
