@@ -196,7 +196,8 @@ static int rowlen_of(int n, int R, const KindGeom& g, size_t elt) {
 // box (45^3 points), 2 orbitals 9.4, 11.1 / 6.5, 7.9; 4 orbitals 11.2, 13.0 / 7.6, 8.1; 8
 // orbitals 17.8, 16.3 / 10.9, 9.0; free 32^3, 8 orbitals 108, 52 / 56, 32; 64 orbitals
 // 453, 283 / 391, 211.  With a density lines of fewer than 32 outputs stay row-wise: a tile
-// has no full warp then (24 outputs, 64 orbitals: 31 against 36).  The compressed passes of
+// has no full warp then (24 outputs, 64 orbitals: 31 against 36); so do small planes, whose
+// tiles and at most GMAX groups are fewer than two per SM.  The compressed passes of
 // less than 5e5 points are row-wise for the same reason: synthesis pass 1 and analysis pass 3
 // on 20x21x31, 2 orbitals 4.3, 6.0 and 5.3, 7.6; 8 orbitals 8.2, 7.0 and 10.2, 8.2; on 37x45x51,
 // 2 orbitals 9.6, 7.9 and 13.8, 8.5.
@@ -204,7 +205,7 @@ template <typename T>
 static bool use_pass32(const PassCall<T>& c) {
     if (sizeof(T) != 4) return false;
     if (c.mode == M_POT) {
-        long long points = 0, longer = 0;
+        long long points = 0, longer = 0, units = 0;
         bool plain = true;
         for (const auto& d : c.segs) {
             int n, N;
@@ -212,9 +213,10 @@ static bool use_pass32(const PassCall<T>& c) {
             const long long v = (long long)n * N * d.s.norb;
             points += v;
             if (d.user_rho == nullptr || n >= 32) longer += v;
+            units += (long long)((N + 31) / 32) * (d.user_rho ? std::min(d.s.norb, GMAX) : d.s.norb);
             plain = plain && d.user_rho == nullptr && d.s.vN1 == 0;
         }
-        return points >= (plain ? 100000 : 500000) && 2 * longer >= points;
+        return points >= (plain ? 100000 : 500000) && 2 * longer >= points && (plain || units >= 2 * num_sms());
     }
     if (c.mode != M_UNCOMP && c.mode != M_COMP) return false;
     long long points = 0;
