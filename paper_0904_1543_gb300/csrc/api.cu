@@ -1032,6 +1032,29 @@ struct StageClock {
 // kinetic = TA3 (T_3, A_3, compression); the analysis stage stays empty.
 // OP_ENERGY runs SYN3, SKM12 without v, POT3 without x and TA3 for <a, T_3 a>
 // alone; OP_DENSITY runs SYN3, SKM12 (t only) and POT3 (rho only).
+// Launch shapes of a plane kernel for the runs of a batch.  A shape of its own is a launch of its
+// own, whose start and tail cost more than the shape gains on few points: below 8e6 (eight
+// planes of 80^2 per SM) a run joins the others, at 256 threads (5 orbitals on 36x56x40 and 14 on
+// 36x32x40 in one plan, 3.2e6 and 5.2e6 points, 258 us in two launches, 242 in one).
+template <typename T>
+static std::vector<FzShape> fz_shapes(int prog, const std::vector<CellRun<T>>& runs) {
+    std::vector<FzShape> shapes;
+    bool mixed = false;
+    for (const auto& r : runs) {
+        shapes.push_back(fz_plane_shape<T>(prog, r.Nf[0], r.Nf[1], (long long)r.norb * r.Nf[2]));
+        mixed = mixed || shapes.back() != shapes.front();
+    }
+    if (!mixed) return shapes;
+    const std::vector<FzShape> own = shapes;
+    for (size_t k = 0; k < runs.size(); ++k) {
+        long long points = 0;   // of this shape
+        for (size_t j = 0; j < runs.size(); ++j)
+            if (!(own[j] != own[k])) points += runs[j].norb * runs[j].P;
+        if (points < 8000000) shapes[k] = FzShape{256, 0};
+    }
+    return shapes;
+}
+
 template <typename T>
 static wvl_status run_fused(int op, std::vector<CellRun<T>>& runs, Prof* prof, cudaStream_t st) {
     static const int kStage[FZ_NPROG] = {ST_SYN, ST_SYN, ST_MF, ST_MFT, ST_KIN};
@@ -1049,6 +1072,8 @@ static wvl_status run_fused(int op, std::vector<CellRun<T>>& runs, Prof* prof, c
         if (!hpsi && prog == FZ_MFTA12) continue;
         if (!energy && prog == FZ_TA3) continue;
         clk.begin(kStage[prog]);
+        std::vector<FzShape> shapes;
+        if (prog == FZ_SKM12 || prog == FZ_MFTA12) shapes = fz_shapes(prog, runs);
         size_t i = 0;
         while (i < runs.size()) {
             FzParams<T> p;
@@ -1075,10 +1100,10 @@ static wvl_status run_fused(int op, std::vector<CellRun<T>>& runs, Prof* prof, c
                 if (k > 0 && (r.hg[0] != r0.hg[0] || r.hg[1] != r0.hg[1] || r.hg[2] != r0.hg[2]))
                     break;
                 const bool plane = prog == FZ_SKM12 || prog == FZ_MFTA12;
-                // one launch shape per launch of a plane kernel
-                const FzShape shape = fz_plane_shape<T>(prog, r.Nf[0], r.Nf[1], (long long)r.norb * r.Nf[2]);
-                if (k > 0 && plane && shape != p.shape) break;
-                p.shape = shape;
+                if (plane) {   // one launch shape per launch of a plane kernel
+                    if (k > 0 && shapes[i] != p.shape) break;
+                    p.shape = shapes[i];
+                }
                 FzSeg<T>& s = p.seg[k];
                 s.P = r.P;
                 s.N1 = r.Nf[0];
