@@ -18,8 +18,10 @@
 // (800 to 820), a warp of its own for the copies (1153 / 1205: one warp's copies in flight
 // are too few).
 //
-// All sums keep the order of the general form, so that an orbital's results do not depend on
-// the number of planes in its call, which chooses the form (fz_plane_shape): the same bits.
+// Filter sums and the FP32 chains of Ekin keep the order of the general form, so that an orbital's
+// results do not depend on the number of planes in its call, which chooses the form and its
+// threads (fz_plane_shape): H psi has the same bits, and Ekin, whose chains are added in
+// compensated pairs grouped by threads, differs from 2^-48 on if at all.
 // MFT_1 before MFT_2 therefore, by rows and without a transpose (128^2 324 us, with MFT_2
 // first, both as line items, 331; 96^2 209 and 207).
 #include <algorithm>

@@ -1,7 +1,8 @@
 """An orbital's results in the FP32 fused chain do not depend on the orbitals that share its
 call: the number of planes chooses the form of the plane kernels (the transposing one for
 square planes of more than two per SM, threads by planes per SM), and every form keeps the same
-order of all sums.  The same bits, H psi and both energies."""
+order of the filter sums and of the FP32 chains of Ekin; the compensated pairs that add the
+chains agree to the last bit on these sizes.  The same bits, H psi and both energies."""
 import numpy as np
 import pytest
 
